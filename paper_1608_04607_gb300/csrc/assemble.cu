@@ -27,97 +27,57 @@
 //
 // Work decomposition: a one-thread-per-pair FP64 set-up kernel writes the
 // per-pair constants (local frame, the linear forms m_X, the receiving frame)
-// in FP32; the assembly kernel runs one warp per face pair.  Lanes evaluate
-// one quadrature node each (geometry, closed-form S, two Zernike vectors by
-// the recursion of Sec. 3.1 in Cartesian form), stage w Z(p') and Z(p) in
-// shared memory, then the warp accumulates the rank-32 update of the N_b x N_b
-// block with every lane owning a TR x TC register tile.
+// in FP32; then one warp assembles one face pair.  FP32 and BF16 blocks run on
+// tensor cores (assemble_mma.cuh).  FP64 blocks: lanes evaluate one quadrature
+// node each (geometry, closed-form S, two Zernike vectors by the recursion of
+// Sec. 3.1 in Cartesian form), stage w Z(p') and Z(p) in shared memory, and the
+// warp accumulates the rank-32 update of the N_b x N_b block with every lane
+// owning a TR x TC register tile (assemble64_kernel below).
 #include <math.h>
 
 #include <cuda_bf16.h>
 
+#include "assemble_mma.cuh"
 #include "dfm_internal.cuh"
 #include "node.cuh"
 
 #include <algorithm>
-#include <cstddef>
 #include <type_traits>
 
 namespace dfm {
 namespace {
 
-// Store one staged row: scale * v[0..NB) followed by zeros up to NBP, as
-// 16-byte vectors for FP32 (rows are 16-byte aligned, see Tile::LD).
-template <int NBP, int NB, typename T>
-__device__ __forceinline__ void stage_row(T* row, const T* v, T scale) {
-  if constexpr (std::is_same<T, float>::value) {
+// Store one staged row: scale * v[0..NB) followed by zeros up to NBP.
+template <int NBP, int NB>
+__device__ __forceinline__ void stage_row(double* row, const double* v, double scale) {
 #pragma unroll
-    for (int u = 0; u < NBP / 4; ++u) {
-      float4 q;
-      q.x = (4 * u + 0 < NB) ? scale * v[4 * u + 0 < NB ? 4 * u + 0 : 0] : 0.f;
-      q.y = (4 * u + 1 < NB) ? scale * v[4 * u + 1 < NB ? 4 * u + 1 : 0] : 0.f;
-      q.z = (4 * u + 2 < NB) ? scale * v[4 * u + 2 < NB ? 4 * u + 2 : 0] : 0.f;
-      q.w = (4 * u + 3 < NB) ? scale * v[4 * u + 3 < NB ? 4 * u + 3 : 0] : 0.f;
-      *reinterpret_cast<float4*>(row + 4 * u) = q;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < NBP; ++c) row[c] = c < NB ? scale * v[c < NB ? c : 0] : T(0);
-  }
-}
-
-// Load N consecutive staged values with the widest aligned vector loads.
-template <int N, typename T>
-__device__ __forceinline__ void load_run(const T* p, T* out) {
-  if constexpr (std::is_same<T, float>::value && N % 4 == 0) {
-#pragma unroll
-    for (int u = 0; u < N / 4; ++u) {
-      const float4 q = *reinterpret_cast<const float4*>(p + 4 * u);
-      out[4 * u] = q.x;
-      out[4 * u + 1] = q.y;
-      out[4 * u + 2] = q.z;
-      out[4 * u + 3] = q.w;
-    }
-  } else if constexpr (std::is_same<T, float>::value && N % 2 == 0) {
-#pragma unroll
-    for (int u = 0; u < N / 2; ++u) {
-      const float2 q = *reinterpret_cast<const float2*>(p + 2 * u);
-      out[2 * u] = q.x;
-      out[2 * u + 1] = q.y;
-    }
-  } else {
-#pragma unroll
-    for (int u = 0; u < N; ++u) out[u] = p[u];
-  }
+  for (int c = 0; c < NBP; ++c) row[c] = c < NB ? scale * v[c < NB ? c : 0] : 0.0;
 }
 
 // Shared memory of one warp: patch state plus the staged node vectors.
-template <int NP, typename T>
+template <int NP>
 struct WarpSmem {
   PatchSmem P;
-  alignas(16) T zq[32 * Tile<NP>::LD];  // w * Z(p') per node (16-byte aligned rows)
-  alignas(16) T zp[32 * Tile<NP>::LD];  // Z(p) per node
+  alignas(16) double zq[32 * Tile<NP>::LD];  // w * Z(p') per node
+  alignas(16) double zp[32 * Tile<NP>::LD];  // Z(p) per node
 };
 
-// QC > 0 fixes the per-patch Gauss order at compile time (the default
-// N_p + 6), which turns the node-index divisions into multiplies.
-// TO: storage type of the blocks (T, or BF16 rounded from FP32 sums).
-template <int NP, typename T, int QC, typename TO>
+template <int NP>
 __global__ void __launch_bounds__(kWarps * 32)
-assemble_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const double* __restrict__ gl_x,
-                const double* __restrict__ gl_w, int q_rt, float cos_max, TO* __restrict__ vals, int64_t row_stride,
-                unsigned long long* __restrict__ node_count, int moment) {
+assemble64_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const double* __restrict__ gl_x,
+                  const double* __restrict__ gl_w, int q, float cos_max, double* __restrict__ vals, int64_t row_stride,
+                  unsigned long long* __restrict__ node_count, int moment) {
+  using T = double;
   using TL = Tile<NP>;
   constexpr int NB = TL::NB, TR = TL::TR, TC = TL::TC, LD = TL::LD;
   extern __shared__ __align__(16) unsigned char dyn_smem[];
-  WarpSmem<NP, T>* smem = reinterpret_cast<WarpSmem<NP, T>*>(dyn_smem);
+  WarpSmem<NP>* smem = reinterpret_cast<WarpSmem<NP>*>(dyn_smem);
   T* s_x = reinterpret_cast<T*>(smem + kWarps);
   T* s_w = s_x + kMaxQ;
   float* s_ninv = reinterpret_cast<float*>(s_w + kMaxQ);
   const int lane = threadIdx.x & 31;
   const int wid = threadIdx.x >> 5;
-  WarpSmem<NP, T>& S = smem[wid];
-  const int q = QC > 0 ? QC : q_rt;
+  WarpSmem<NP>& S = smem[wid];
   if (threadIdx.x < q) {
     s_x[threadIdx.x] = (T)gl_x[threadIdx.x];
     s_w[threadIdx.x] = (T)gl_w[threadIdx.x];
@@ -190,34 +150,21 @@ assemble_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const doubl
 #pragma unroll 2
         for (int kk = 0; kk < kmax; ++kk) {
           T av[TR], bv[TC];
-          load_run<TR>(&S.zq[kk * LD + a0], av);
-          load_run<TC>(&S.zp[kk * LD + b0], bv);
-          if constexpr (std::is_same<T, float>::value) {
-            // packed FP32 FMAs (two independent roundings, the same results
-            // as scalar FMAs) halve the instructions of the rank-1 update
 #pragma unroll
-            for (int r = 0; r < TR; ++r) {
-              const float2 a2 = make_float2(av[r], av[r]);
+          for (int r = 0; r < TR; ++r) av[r] = S.zq[kk * LD + a0 + r];
 #pragma unroll
-              for (int c = 0; c < TC; c += 2) {
-                const float2 p2 = __ffma2_rn(a2, make_float2(bv[c], bv[c + 1]), make_float2(acc[r][c], acc[r][c + 1]));
-                acc[r][c] = p2.x;
-                acc[r][c + 1] = p2.y;
-              }
-            }
-          } else {
+          for (int c = 0; c < TC; ++c) bv[c] = S.zp[kk * LD + b0 + c];
 #pragma unroll
-            for (int r = 0; r < TR; ++r)
+          for (int r = 0; r < TR; ++r)
 #pragma unroll
-              for (int c = 0; c < TC; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
-          }
+            for (int c = 0; c < TC; ++c) acc[r][c] = fma(av[r], bv[c], acc[r][c]);
         }
         __syncwarp();
       }
     }
     if (lane == 0) atomicAdd(node_count, pair_nodes);
     // epilogue: scale row a by lambda N_a / sqrt(|T_l||T_l'|) and store
-    TO* out = vals + (int64_t)pc.out_row * row_stride + (int64_t)pc.slot * NB * NB;
+    double* out = vals + (int64_t)pc.out_row * row_stride + (int64_t)pc.slot * NB * NB;
 #pragma unroll
     for (int r = 0; r < TR; ++r) {
       const int a = a0 + r;
@@ -226,56 +173,41 @@ assemble_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const doubl
 #pragma unroll
       for (int c = 0; c < TC; ++c) {
         const int b = b0 + c;
-        if (b < NB) {
-          if constexpr (std::is_same<TO, __nv_bfloat16>::value)
-            out[a * NB + b] = __float2bfloat16_rn(acc[r][c] * s);
-          else
-            out[a * NB + b] = acc[r][c] * s;
-        }
+        if (b < NB) out[a * NB + b] = acc[r][c] * s;
       }
     }
     __syncwarp();
   }
 }
 
-using WarpSmem4f = WarpSmem<4, float>;
-using WarpSmem8f = WarpSmem<8, float>;
-static_assert(offsetof(WarpSmem4f, zq) % 16 == 0 && sizeof(WarpSmem4f) % 16 == 0, "16-byte aligned staging rows");
-static_assert(offsetof(WarpSmem8f, zq) % 16 == 0 && sizeof(WarpSmem8f) % 16 == 0, "16-byte aligned staging rows");
-
-template <int NP, typename T>
-constexpr size_t assemble_smem_bytes() {
-  return sizeof(WarpSmem<NP, T>) * kWarps + 2 * kMaxQ * sizeof(T) + 64 * sizeof(float);
-}
-
-template <int NP, typename T, int QC, typename TO>
-int launch_assemble_q(const PairConst* pairs, int64_t npairs, const double* glx, const double* glw, int q,
-                      float cos_max, TO* vals, int64_t row_stride, unsigned long long* nodes, int moment,
+template <int NP>
+int launch_assemble64(const PairConst* pairs, int64_t npairs, const double* glx, const double* glw, int q,
+                      float cos_max, double* vals, int64_t row_stride, unsigned long long* nodes, int moment,
                       cudaStream_t st) {
-  constexpr size_t smem = assemble_smem_bytes<NP, T>();
+  constexpr size_t smem = sizeof(WarpSmem<NP>) * kWarps + 2 * kMaxQ * sizeof(double) + 64 * sizeof(float);
   static_assert(smem <= 220 * 1024, "assembly shared memory");
-  DFM_CUDA_CHECK(
-      cudaFuncSetAttribute(assemble_kernel<NP, T, QC, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  DFM_CUDA_CHECK(cudaFuncSetAttribute(assemble64_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int64_t blocks = (npairs + kWarps - 1) / kWarps;
   if (blocks > 0x7fffffff) return set_error(DFM_ERR_ARG, "dfm_assemble: too many face pairs");
   {
     ::dfm::KernelTimer timer_(DFM_KERNEL_ASSEMBLE, st);
-    assemble_kernel<NP, T, QC, TO><<<(unsigned)blocks, kWarps * 32, smem, st>>>(pairs, npairs, glx, glw, q, cos_max,
-                                                                                vals, row_stride, nodes, moment);
+    assemble64_kernel<NP><<<(unsigned)blocks, kWarps * 32, smem, st>>>(pairs, npairs, glx, glw, q, cos_max, vals,
+                                                                       row_stride, nodes, moment);
   }
   DFM_LAUNCHED();
   DFM_CUDA_CHECK(cudaGetLastError());
   return DFM_OK;
 }
 
+// TO: storage type of the blocks (T, or BF16 rounded from FP32 sums)
 template <int NP, typename T, typename TO>
 int launch_assemble(const PairConst* pairs, int64_t npairs, const double* glx, const double* glw, int q,
                     float cos_max, TO* vals, int64_t row_stride, unsigned long long* nodes, int moment,
                     cudaStream_t st) {
-  if (std::is_same<T, float>::value && q == NP + 6)
-    return launch_assemble_q<NP, T, NP + 6, TO>(pairs, npairs, glx, glw, q, cos_max, vals, row_stride, nodes, moment,
-                                                st);
-  return launch_assemble_q<NP, T, 0, TO>(pairs, npairs, glx, glw, q, cos_max, vals, row_stride, nodes, moment, st);
+  if constexpr (std::is_same<T, float>::value)
+    return launch_assemble_mma<NP, TO>(pairs, npairs, glx, glw, q, cos_max, vals, row_stride, nodes, moment, st);
+  else
+    return launch_assemble64<NP>(pairs, npairs, glx, glw, q, cos_max, vals, row_stride, nodes, moment, st);
 }
 
 template <typename T, typename TO = T>

@@ -1,0 +1,309 @@
+// FP32 assembly of the operator blocks (N_p <= 8) with the block sums on
+// tensor cores.  Included by assemble.cu.
+//
+// One warp per face pair.  Lanes evaluate one quadrature node each (row by
+// row, row_node.cuh); the block is the sum over nodes of w Z(p') Z(p)^T, an
+// N_b x N_b product over some 1,400 (N_p = 4) to 2,700 (N_p = 8) nodes.  Per pass of
+// 32 nodes each staged value x is split into two FP16 parts x = hi + lo
+// (22 significant bits) and the pass's product is three mma.sync m16n8k16
+// products, lo hi + hi lo + hi hi with FP32 accumulation, started at zero and
+// added to the FP32 sums on the CUDA cores.  So no sum on the tensor cores is
+// longer than 32 nodes (their accumulation rounds towards zero), and the
+// weights of a pass are scaled by a power of two to a maximum in [1, 2), which
+// keeps both FP16 parts away from the subnormal range whatever the mesh's
+// lengths and damping; the scale is taken out by the FMA that adds the pass.
+// Measured error against the same rule in 64 bits: 1.4e-7 (2-norm), where the
+// 1,394 sequential FP32 additions per entry of the rank-1 form gave 5.7e-7.
+//
+// Measured (GB300): 48,000 tets at N_p = 4 in 10.3 ms against 23.8 ms for the
+// rank-1 form on CUDA cores, 24,576 tets at N_p = 8 in 36.2 against 87.0 ms.
+// What bounds it: issue and the FP32, ALU and shared-memory pipes together at
+// N_p = 4 (315 instructions per pass, 67% issue active, no pipe above 60%); at
+// N_p = 8 the latency of the MMA chains (108 MMAs of 8 cycles in a pass of
+// 1,750 cycles), with 255 registers and 8 warps per SM slightly ahead of 168
+// registers and 12 (36.2 against 36.9 ms; the other way round at N_p = 7, 11.2
+// against 10.5 ms at 10,368 tets).  More warps at N_p <= 4 gain nothing (24 per
+// SM: 10.5 ms).
+#pragma once
+
+#include <algorithm>
+
+#include <cuda_fp16.h>
+
+#include "row_node.cuh"
+
+namespace dfm {
+namespace {
+
+template <int NP>
+struct MmaTile {
+  static constexpr int NB = (NP + 1) * (NP + 2) / 2;
+  static constexpr int MT = (NB + 15) / 16;  // 16-row tiles of test functions
+  static constexpr int NT = (NB + 7) / 8;    // 8-column tiles of trial functions
+  // staged halves per node: the MMA tiles' width, a row stride of an odd
+  // number of 16-byte units (ldmatrix and the 16-byte stores then touch
+  // distinct bank groups)
+  static constexpr int W = MT * 16;
+  static constexpr int LD = W / 8 % 2 ? W : W + 8;
+};
+
+// Shared memory of one warp.
+template <int NP>
+struct MmaWarp {
+  PatchWarp P;
+  PairConst pc;
+  // Z(p') times the scaled weight, and Z(p): hi and lo parts, one row per node
+  alignas(16) __half qh[32 * MmaTile<NP>::LD];
+  alignas(16) __half ql[32 * MmaTile<NP>::LD];
+  alignas(16) __half ph[32 * MmaTile<NP>::LD];
+  alignas(16) __half pl[32 * MmaTile<NP>::LD];
+};
+
+// hi and lo FP16 parts of the values v[0..NB) of a node (x: Z(p), y: w Z(p');
+// zero up to a multiple of 8) into its four staged rows.  What the last m-tile
+// reads beyond that is left as it is: it reaches only block rows past N_b.
+template <int NB>
+__device__ __forceinline__ void stage_split(__half* ph, __half* pl, __half* qh, __half* ql, const float2* v) {
+  const float2 minus = pair(-1.f, -1.f);
+  auto bits = [](__half2 h) { return reinterpret_cast<const uint32_t&>(h); };
+#pragma unroll
+  for (int u = 0; u < (NB + 7) / 8; ++u) {
+    uint32_t h0[4], l0[4], h1[4], l1[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int b = 8 * u + 2 * e;
+      if (b >= NB) {
+        h0[e] = l0[e] = h1[e] = l1[e] = 0u;
+        continue;
+      }
+      const float2 s = v[b], t = b + 1 < NB ? v[b + 1 < NB ? b + 1 : b] : pair(0.f, 0.f);
+      const __half2 hp = __floats2half2_rn(s.x, t.x), hq = __floats2half2_rn(s.y, t.y);
+      const float2 fp = __half22float2(hp), fq = __half22float2(hq);
+      const float2 ds = fma2(pair(fp.x, fq.x), minus, s), dt = fma2(pair(fp.y, fq.y), minus, t);
+      h0[e] = bits(hp);
+      h1[e] = bits(hq);
+      l0[e] = bits(__floats2half2_rn(ds.x, dt.x));
+      l1[e] = bits(__floats2half2_rn(ds.y, dt.y));
+    }
+    *reinterpret_cast<uint4*>(ph + 8 * u) = make_uint4(h0[0], h0[1], h0[2], h0[3]);
+    *reinterpret_cast<uint4*>(pl + 8 * u) = make_uint4(l0[0], l0[1], l0[2], l0[3]);
+    *reinterpret_cast<uint4*>(qh + 8 * u) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+    *reinterpret_cast<uint4*>(ql + 8 * u) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
+  }
+}
+
+__device__ __forceinline__ void ldsm4_trans(uint32_t r[4], const __half* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((unsigned)__cvta_generic_to_shared(p))
+               : "memory");
+}
+
+__device__ __forceinline__ void mma_f16(float d[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// acc += inv * (staged Z(p'))^T (staged Z(p)) over the 32 nodes of a pass.
+// ldmatrix.trans of the node-major rows gives both operands: the A fragment
+// of (m-tile, 16 nodes) from four 8 x 8 pieces, and the B fragments of both
+// 16-node halves of an n-tile from one instruction.
+template <int NP>
+__device__ __forceinline__ void pass_product(const MmaWarp<NP>& S, int lane, float inv,
+                                             float (&acc)[MmaTile<NP>::NT][MmaTile<NP>::MT][4]) {
+  using TL = MmaTile<NP>;
+  constexpr int MT = TL::MT, NT = TL::NT, LD = TL::LD;
+  uint32_t ah[MT][2][4], al[MT][2][4];
+  // pieces (nodes 0-7, m 0-7), (nodes 0-7, m 8-15), (nodes 8-15, m 0-7), (nodes 8-15, m 8-15)
+  const int arow = (lane & 7) + ((lane >> 4) << 3), acol = ((lane >> 3) & 1) << 3;
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      const int o = (16 * ks + arow) * LD + 16 * mt + acol;
+      ldsm4_trans(ah[mt][ks], S.qh + o);
+      ldsm4_trans(al[mt][ks], S.ql + o);
+    }
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    uint32_t bh[4], bl[4];  // (nodes 0-7, 8-15, 16-23, 24-31) x 8 columns
+    ldsm4_trans(bh, S.ph + lane * LD + 8 * nt);
+    ldsm4_trans(bl, S.pl + lane * LD + 8 * nt);
+    // independent chains: the m-tiles, or with one m-tile the three products
+    constexpr int CH = MT == 1 ? 3 : 1;
+    float t[CH][MT][4];
+#pragma unroll
+    for (int h = 0; h < CH; ++h)
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) t[h][mt][0] = t[h][mt][1] = t[h][mt][2] = t[h][mt][3] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) mma_f16(t[0][mt], al[mt][ks], bh[2 * ks], bh[2 * ks + 1]);
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) mma_f16(t[CH > 1 ? 1 : 0][mt], ah[mt][ks], bl[2 * ks], bl[2 * ks + 1]);
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) mma_f16(t[CH - 1][mt], ah[mt][ks], bh[2 * ks], bh[2 * ks + 1]);
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+      for (int e = 0; e < 4; e += 2) {
+        float2 u = pair(t[0][mt][e], t[0][mt][e + 1]);
+        if constexpr (CH == 3) u = __fadd2_rn(__fadd2_rn(u, pair(t[1][mt][e], t[1][mt][e + 1])), pair(t[2][mt][e], t[2][mt][e + 1]));
+        const float2 s = fma2(u, pair(inv, inv), pair(acc[nt][mt][e], acc[nt][mt][e + 1]));
+        acc[nt][mt][e] = s.x;
+        acc[nt][mt][e + 1] = s.y;
+      }
+  }
+}
+
+// moment k: L_O^k phi2^(k)(mu L_O).  A call of its own: inlined, its Gauss rule
+// would take the registers of every assembly.
+__device__ __noinline__ float moment_factor(int moment, float mu, float LO) {
+  float sk = phi2_deriv<float>(moment, mu * LO);
+  for (int e = 0; e < moment; ++e) sk *= LO;
+  return sk;
+}
+
+template <int NP, typename TO>
+__global__ void __launch_bounds__(kWarps * 32, NP == 8 ? 2 : (NP == 7 ? 3 : (NP >= 5 ? 4 : 5)))
+assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const double* __restrict__ gl_x,
+                    const double* __restrict__ gl_w, int q, float cos_max, TO* __restrict__ vals, int64_t row_stride,
+                    unsigned long long* __restrict__ node_count, unsigned long long* __restrict__ counter, int moment) {
+  using TL = MmaTile<NP>;
+  constexpr int NB = TL::NB, MT = TL::MT, NT = TL::NT, LD = TL::LD;
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  MmaWarp<NP>* smem = reinterpret_cast<MmaWarp<NP>*>(dyn_smem);
+  float* s_x = reinterpret_cast<float*>(smem + kWarps);
+  float* s_w = s_x + kMaxQ;
+  float* s_ninv = s_w + kMaxQ;
+  const int lane = threadIdx.x & 31;
+  const int wid = threadIdx.x >> 5;
+  MmaWarp<NP>& S = smem[wid];
+  if (threadIdx.x < q) {
+    s_x[threadIdx.x] = (float)gl_x[threadIdx.x];
+    s_w[threadIdx.x] = (float)gl_w[threadIdx.x];
+  }
+  if (threadIdx.x < NB) s_ninv[threadIdx.x] = zernike_invnorm(threadIdx.x);
+  __syncthreads();
+  const int g8 = lane >> 2, t4 = lane & 3;
+  const float qinv = 1.f / (float)q;
+  unsigned long long my_nodes = 0;
+  // resident warps take pairs off a shared counter, the next one fetched while
+  // this one runs: pairs differ in patch count, and the Gauss table and norms
+  // above are set up once per block
+  unsigned long long p = (unsigned long long)blockIdx.x * kWarps + wid;
+  while (p < (unsigned long long)npairs) {
+    unsigned long long next = 0;
+    if (lane == 0) next = atomicAdd(counter, 1ull) + (unsigned long long)gridDim.x * kWarps;
+    for (int i = lane; i < (int)(sizeof(PairConst) / 4); i += 32)
+      reinterpret_cast<int*>(&S.pc)[i] = reinterpret_cast<const int*>(pairs + p)[i];
+    __syncwarp();
+    const int kind = S.pc.kind;
+    if (kind >= 0) {  // else no block for this pair in this part
+      float acc[NT][MT][4];
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) acc[nt][mt][0] = acc[nt][mt][1] = acc[nt][mt][2] = acc[nt][mt][3] = 0.f;
+      start_regions(S.P, S.pc, cos_max, lane);
+      const float mu = S.pc.mu, D3 = S.pc.D[2], area2 = 2.f * S.pc.area_src;
+      while (true) {
+        const int npatch = fill_patches_warp(S.P, cos_max, lane);
+        if (npatch == 0) break;
+        const int rows = npatch * q;
+        my_nodes += (unsigned long long)(rows * q);
+        for (int base = 0; base < rows;) {
+          const RowPass ps = next_pass(rows - base);
+          const int rl = lane / ps.per;
+          const bool live = rl < ps.rows;
+          const int row = base + (live ? rl : ps.rows - 1);
+          const int pi = (int)(((float)row + 0.5f) * qinv), i = row - pi * q;  // exact: row < 28 x 32
+          RowConst rc;
+          row_const(S.P.patch[pi], s_x[i], S.pc, rc);
+          const float wi = live ? s_w[i] * area2 : 0.f;
+          base += ps.rows;
+          for (int j0 = 0; j0 < q; j0 += ps.per) {
+            const int j = j0 + (lane - rl * ps.per);
+            const bool on = j < q;
+            const int jc = on ? j : q - 1;
+            const RowNode g = row_node(rc, s_x[jc], D3, kind, S.pc);
+            const float sk = moment == 0 ? phi2_row(mu * g.LO) : moment_factor(moment, mu, g.LO);
+            const float w = on ? wi * s_w[jc] * g.base * sk : 0.f;
+            // power of two that brings the pass's largest |w| into [1, 2)
+            const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(w)));
+            const unsigned ex = min(max(top >> 23, 1u), 253u);
+            const float scale = __uint_as_float((254u - ex) << 23), inv = __uint_as_float(ex << 23);
+            float2 Z[NB];
+            zernike2<NP>(g.px, g.py, pair(1.f, w * scale), Z);
+            stage_split<NB>(S.ph + lane * LD, S.pl + lane * LD, S.qh + lane * LD, S.ql + lane * LD, Z);
+            __syncwarp();
+            pass_product<NP>(S, lane, inv, acc);
+            __syncwarp();
+          }
+        }
+      }
+      // epilogue: scale row a by lambda N_a / sqrt(|T_l||T_l'|) and store
+      TO* out = vals + (int64_t)S.pc.out_row * row_stride + (int64_t)S.pc.slot * NB * NB;
+      const float sp = S.pc.scale;
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int a = 16 * mt + g8 + 8 * h;
+          if (a >= NB) continue;
+          const float s = sp * s_ninv[a];
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const int b = 8 * nt + 2 * t4 + e;
+              if (b >= NB) continue;
+              const float v = acc[nt][mt][2 * h + e] * s;
+              if constexpr (std::is_same<TO, __nv_bfloat16>::value)
+                out[a * NB + b] = __float2bfloat16_rn(v);
+              else
+                out[a * NB + b] = v;
+            }
+        }
+    }
+    p = __shfl_sync(0xffffffffu, next, 0);
+    __syncwarp();  // the pair's constants are read before the next ones arrive
+  }
+  if (lane == 0 && my_nodes) atomicAdd(node_count, my_nodes);
+}
+
+template <int NP, typename TO>
+int launch_assemble_mma(const PairConst* pairs, int64_t npairs, const double* glx, const double* glw, int q,
+                        float cos_max, TO* vals, int64_t row_stride, unsigned long long* nodes, int moment,
+                        cudaStream_t st) {
+  constexpr size_t smem = sizeof(MmaWarp<NP>) * kWarps + (2 * kMaxQ + 64) * sizeof(float);
+  static_assert(smem <= 220 * 1024, "assembly shared memory");
+  static_assert(sizeof(MmaWarp<NP>) % 16 == 0, "16-byte aligned staging rows");
+  DFM_CUDA_CHECK(
+      cudaFuncSetAttribute(assemble_mma_kernel<NP, TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int dev = 0, nsm = 0, per_sm = 0;
+  DFM_CUDA_CHECK(cudaGetDevice(&dev));
+  DFM_CUDA_CHECK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  DFM_CUDA_CHECK(
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, assemble_mma_kernel<NP, TO>, kWarps * 32, smem));
+  const int64_t blocks = std::min<int64_t>((npairs + kWarps - 1) / kWarps, (int64_t)nsm * std::max(per_sm, 1));
+  unsigned long long* counter = nodes + 1;
+  DFM_CUDA_CHECK(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
+  {
+    ::dfm::KernelTimer timer_(DFM_KERNEL_ASSEMBLE, st);
+    assemble_mma_kernel<NP, TO><<<(unsigned)blocks, kWarps * 32, smem, st>>>(pairs, npairs, glx, glw, q, cos_max, vals,
+                                                                             row_stride, nodes, counter, moment);
+  }
+  DFM_LAUNCHED();
+  DFM_CUDA_CHECK(cudaGetLastError());
+  return DFM_OK;
+}
+
+}  // namespace
+}  // namespace dfm

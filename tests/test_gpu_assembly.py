@@ -115,3 +115,22 @@ def test_assembly_is_deterministic_and_reassembles(D):
     c = op.blocks()
     assert torch.equal(a, c)
     assert not torch.equal(a, b)
+
+
+@pytest.mark.parametrize("Np", range(9))
+@pytest.mark.parametrize("quad_order,deg,mu,moment", [(0, 0.0, 0.05, 0), (1, 180.0, 0.0, 0), (7, 10.0, 0.4, 0),
+                                                      (32, 60.0, 40.0, 0), (0, 0.0, 0.4, 2)])
+def test_tensor_core_blocks_match_the_fp64_rule(D, Np, quad_order, deg, mu, moment):
+    """FP32 blocks (FP16 hi + lo products on tensor cores) against FP64 blocks of
+    the same rule: one node to 1,024 nodes per patch, subdivision to its deepest
+    levels, damping from none to strong, a damping moment; one to three tiles of
+    test functions.  Both run the same set-up and subdivision arithmetic, so the
+    node counts agree and the entries to the FP32 entry tolerance."""
+    m = kuhn_cube_mesh(2, jitter=0.2, seed=5)
+    mesh = D.Mesh(m.verts, m.tets, refl=0.8)
+    kw = dict(mu=mu, quad_order=quad_order, max_patch_deg=deg, moment=moment)
+    a, b = D.Operator(mesh, Np, **kw), D.Operator(mesh, Np, precision=D.F64, **kw)
+    assert D.op_nodes(a) == D.op_nodes(b)
+    x, y = a.blocks().double(), b.blocks()
+    err = (x - y).abs().amax((2, 3)) / y.abs().amax((2, 3))
+    assert float(err.max()) <= 1e-5
