@@ -643,9 +643,9 @@ extern "C" int dfm_adjoint(const dfm_op* op, const dfm_params* params, const dou
   if (media != (op->rop != nullptr))
     return set_error(DFM_ERR_ARG, "dfm_adjoint: params->c / rho_f differ from the operator's assembly");
   for (int part = 0; part < (media ? 2 : 1); ++part) {
-    pair_setup_kernel<<<(unsigned)((npairs + 127) / 128), 128, 0, st>>>(mesh->verts, mesh->tets, mesh->recv,
+    pair_setup_kernel<<<(unsigned)((mesh->nrows + 127) / 128), 128, 0, st>>>(mesh->verts, mesh->tets, mesh->recv,
                                                                        mesh->refl, mesh->geom, params->mu,
-                                                                       params->mu_uniform, npairs, pairs, params->c,
+                                                                       params->mu_uniform, mesh->nrows, pairs, params->c,
                                                                        params->rho_f, part);
     DFM_LAUNCHED();
     DFM_CUDA_CHECK(cudaGetLastError());

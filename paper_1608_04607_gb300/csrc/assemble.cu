@@ -346,9 +346,9 @@ extern "C" int dfm_assemble_into(const dfm_mesh* mesh, const dfm_params* p, dfm_
   for (int part = 0; part < (media ? 2 : 1); ++part) {
     dfm_op* dst = part == 0 ? op : op->rop;
     if (part == 1) DFM_CUDA_CHECK(cudaMemsetAsync(dst->vals, 0, dst->bytes, st));  // non-interface blocks stay 0
-    pair_setup_kernel<<<(unsigned)((npairs + bs - 1) / bs), bs, 0, st>>>(mesh->verts, mesh->tets, mesh->recv,
+    pair_setup_kernel<<<(unsigned)((mesh->nrows + bs - 1) / bs), bs, 0, st>>>(mesh->verts, mesh->tets, mesh->recv,
                                                                          mesh->refl, mesh->geom, p->mu,
-                                                                         p->mu_uniform, npairs, pairs, p->c,
+                                                                         p->mu_uniform, mesh->nrows, pairs, p->c,
                                                                          p->rho_f, part);
     DFM_LAUNCHED();
     DFM_CUDA_CHECK(cudaGetLastError());

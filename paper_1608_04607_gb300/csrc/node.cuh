@@ -78,7 +78,10 @@ __device__ __forceinline__ double dot3(const double* a, const double* b) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-// One thread per face pair p = 12 t + 3 f + k (k-th destination face l' != f).
+// Pairs p = 12 t + 3 f + k (k-th destination face l' != f), one thread per
+// source face (t, f): the tet's vertices in the face frame and the three
+// barycentric forms of the face serve its three pairs, which differ only in
+// which face vertex is A.  FP64 issue bounds it (two lanes per SM).
 // c_tet, rhof_tet: per-tet speed and fluid density (NULL: 1).  part 0: the
 // blocks received across l' (transmitted, or reflected at the boundary);
 // part 1: the blocks reflected at an interface between different media, kind
@@ -86,89 +89,91 @@ __device__ __forceinline__ double dot3(const double* a, const double* b) {
 __global__ void pair_setup_kernel(const double* __restrict__ V, const int32_t* __restrict__ tets,
                                   const int32_t* __restrict__ recv, const double* __restrict__ refl,
                                   const FaceGeom* __restrict__ geom, const double* __restrict__ mu_tet,
-                                  double mu_uniform, int64_t npairs, PairConst* __restrict__ out,
+                                  double mu_uniform, int64_t nfaces, PairConst* __restrict__ out,
                                   const double* __restrict__ c_tet = nullptr,
                                   const double* __restrict__ rhof_tet = nullptr, int part = 0) {
-  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= npairs) return;
-  const int64_t t = p / 12;
-  const int f = (int)((p % 12) / 3);
-  const int k = (int)(p % 3);
-  const int fp = k + (k >= f ? 1 : 0);
-  const FaceGeom g = geom[4 * t + f];
+  const int64_t row = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (row >= nfaces) return;
+  const int64_t t = row >> 2;
+  const int f = (int)(row & 3);
+  const FaceGeom g = geom[row];
   const int32_t* tv = tets + 4 * t;
-  // local coordinates of the tet's vertices
-  double loc[4][3];
-  for (int v = 0; v < 4; ++v) {
+  // local coordinates of the face's vertices (f + 1, f + 2, f + 3) mod 4 and of D = vertex f
+  double P[3][3], D[3];
+  auto local = [&](int v, double* o) {
     double r[3];
     for (int c = 0; c < 3; ++c) r[c] = V[3 * (int64_t)tv[v] + c] - g.o[c];
-    loc[v][0] = dot3(r, g.e1);
-    loc[v][1] = dot3(r, g.e2);
-    loc[v][2] = dot3(r, g.n);
-  }
-  // A = vertex fp (on the source face), B, C the other two face vertices in face order, D = vertex f
-  int bc[2], nb = 0;
-  for (int j = 1; j <= 3; ++j) {
-    const int v = (f + j) & 3;
-    if (v != fp) bc[nb++] = v;
-  }
-  const double* A = loc[fp];
-  const double* B = loc[bc[0]];
-  const double* C = loc[bc[1]];
-  const double* D = loc[f];
-  const double D3 = D[2];
-  // m_X = (-D3 grad beta_X, beta_X(D')) for the in-plane barycentric coordinate beta_X
-  auto mvec = [&](const double* X, const double* Y, const double* Z, float* m) {
-    const double zy0 = Z[0] - Y[0], zy1 = Z[1] - Y[1];
-    const double den = zy0 * (X[1] - Y[1]) - zy1 * (X[0] - Y[0]);
-    const double gx = -zy1 / den, gy = zy0 / den;
-    const double betaD = (zy0 * (D[1] - Y[1]) - zy1 * (D[0] - Y[0])) / den;
-    m[0] = (float)(-D3 * gx);
-    m[1] = (float)(-D3 * gy);
-    m[2] = (float)betaD;
+    o[0] = dot3(r, g.e1);
+    o[1] = dot3(r, g.e2);
+    o[2] = dot3(r, g.n);
   };
-  PairConst pc;
-  mvec(A, B, C, pc.mA);
-  mvec(B, C, A, pc.mB);
-  mvec(C, A, B, pc.mC);
-  const int32_t R0 = recv[4 * t + fp];
-  const bool boundary = (R0 == 4 * t + fp);
-  // media of the tet and of the neighbour across l'
-  const int64_t ti = R0 / 4;
-  const double cj = c_tet ? c_tet[t] : 1.0, ci = c_tet ? c_tet[ti] : 1.0;
-  const double zj = cj * (rhof_tet ? rhof_tet[t] : 1.0), zi = ci * (rhof_tet ? rhof_tet[ti] : 1.0);
-  const bool interface = !boundary && (ci != cj || zi != zj);
-  // part 1 blocks are received by face l' of the tet itself
-  const int32_t R = part == 1 ? (int32_t)(4 * t + fp) : R0;
-  const FaceGeom gr = geom[R];
-  pc.R1[0] = (float)dot3(gr.e1, g.e1);
-  pc.R1[1] = (float)dot3(gr.e1, g.e2);
-  pc.R1[2] = (float)dot3(gr.e1, g.n);
-  pc.R2[0] = (float)dot3(gr.e2, g.e1);
-  pc.R2[1] = (float)dot3(gr.e2, g.e2);
-  pc.R2[2] = (float)dot3(gr.e2, g.n);
-  for (int c = 0; c < 3; ++c) {
-    pc.A[c] = (float)A[c];
-    pc.B[c] = (float)B[c];
-    pc.C[c] = (float)C[c];
-    pc.D[c] = (float)D[c];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) local((f + 1 + j) & 3, P[j]);
+  local(f, D);
+  // m_X = (-D3 grad beta_X, beta_X(D')) for the in-plane barycentric coordinate beta_X
+  float m[3][3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const double *X = P[j], *Y = P[(j + 1) % 3], *Z = P[(j + 2) % 3];
+    const double zy0 = Z[0] - Y[0], zy1 = Z[1] - Y[1];
+    const double rden = 1.0 / (zy0 * (X[1] - Y[1]) - zy1 * (X[0] - Y[0]));
+    m[j][0] = (float)(D[2] * zy1 * rden);
+    m[j][1] = (float)(-D[2] * zy0 * rden);
+    m[j][2] = (float)((zy0 * (D[1] - Y[1]) - zy1 * (D[0] - Y[0])) * rden);
   }
-  pc.area_src = (float)g.area;
-  pc.mu = (float)(mu_tet ? mu_tet[t] : mu_uniform);
-  const double lam = boundary ? refl[R] : 1.0;
-  pc.scale = (float)(lam / sqrt(g.area * geom[4 * t + fp].area));
-  pc.out_row = R;
-  pc.slot = f - (f > fp ? 1 : 0);
-  const FaceGeom gd = geom[4 * t + fp];
-  pc.ndst[0] = (float)dot3(gd.n, g.e1);
-  pc.ndst[1] = (float)dot3(gd.n, g.e2);
-  pc.ndst[2] = (float)dot3(gd.n, g.n);
-  pc.c_ratio = (float)(ci / cj);
-  pc.z_src = (float)zj;
-  pc.z_dst = (float)zi;
-  pc.qscale = (part == 0 && interface) ? (float)(ci / cj) : 1.f;
-  pc.kind = part == 0 ? (interface ? 1 : 0) : (interface ? 2 : -1);
-  out[p] = pc;
+  const double cj = c_tet ? c_tet[t] : 1.0;
+  const double zj = cj * (rhof_tet ? rhof_tet[t] : 1.0);
+  const float mu = (float)(mu_tet ? mu_tet[t] : mu_uniform);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {  // A = face vertex a, the one opposite l'; B, C the other two in face order
+    const int fp = (f + 1 + a) & 3;
+    const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
+    PairConst pc;
+#pragma unroll
+    for (int x = 0; x < 3; ++x) {
+      pc.mA[x] = m[a][x];
+      pc.mB[x] = m[b][x];
+      pc.mC[x] = m[c][x];
+      pc.A[x] = (float)P[a][x];
+      pc.B[x] = (float)P[b][x];
+      pc.C[x] = (float)P[c][x];
+      pc.D[x] = (float)D[x];
+    }
+    const int32_t R0 = recv[4 * t + fp];
+    const bool boundary = (R0 == 4 * t + fp);
+    // media of the tet and of the neighbour across l'
+    const int64_t ti = R0 / 4;
+    const double ci = c_tet ? c_tet[ti] : 1.0;
+    const double zi = ci * (rhof_tet ? rhof_tet[ti] : 1.0);
+    const bool interface = !boundary && (ci != cj || zi != zj);
+    // part 1 blocks are received by face l' of the tet itself
+    const int32_t R = part == 1 ? (int32_t)(4 * t + fp) : R0;
+    const FaceGeom gr = geom[R];
+    pc.R1[0] = (float)dot3(gr.e1, g.e1);
+    pc.R1[1] = (float)dot3(gr.e1, g.e2);
+    pc.R1[2] = (float)dot3(gr.e1, g.n);
+    pc.R2[0] = (float)dot3(gr.e2, g.e1);
+    pc.R2[1] = (float)dot3(gr.e2, g.e2);
+    pc.R2[2] = (float)dot3(gr.e2, g.n);
+    const FaceGeom gd = geom[4 * t + fp];
+    pc.area_src = (float)g.area;
+    pc.mu = mu;
+    const double lam = boundary ? refl[R] : 1.0;
+    pc.scale = (float)(lam / sqrt(g.area * gd.area));
+    pc.out_row = R;
+    pc.slot = f - (f > fp ? 1 : 0);
+    pc.ndst[0] = (float)dot3(gd.n, g.e1);
+    pc.ndst[1] = (float)dot3(gd.n, g.e2);
+    pc.ndst[2] = (float)dot3(gd.n, g.n);
+    const float ratio = ci == cj ? 1.f : (float)(ci / cj);
+    pc.c_ratio = ratio;
+    pc.z_src = (float)zj;
+    pc.z_dst = (float)zi;
+    pc.qscale = (part == 0 && interface) ? ratio : 1.f;
+    pc.kind = part == 0 ? (interface ? 1 : 0) : (interface ? 2 : -1);
+    // pair 12 t + 3 f + k, k the rank of l' among the faces other than f
+    out[12 * t + 3 * f + fp - (fp > f ? 1 : 0)] = pc;
+  }
 }
 
 // ---------------------------------------------------------------------------
