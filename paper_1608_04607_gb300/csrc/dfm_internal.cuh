@@ -172,6 +172,12 @@ void destroy_hop_graphs(dfm_op* op);
 // right-hand sides (spmv_mma.cu)
 bool apply_mma_supported(const dfm_op* op, int R);
 int apply_mma(const dfm_op* op, const float* x, const float* x0, float* y, int R, double alpha, cudaStream_t st);
+// tensor-core forward application of K FP32 operators (combo_ops and coef NULL:
+// op alone) to R FP32 right-hand sides (spmv_multi.cu), and whether it is the
+// faster one for this basis, K and R
+bool apply_multi_supported(const dfm_op* op, int K, int R);
+int apply_multi(const dfm_op* op, const dfm_op* const* combo_ops, int K, const double* coef, const float* x,
+                const float* x0, float* y, int R, double alpha, cudaStream_t st);
 // reads and clears op's time-out flag (waits on st): DFM_ERR_TIMEOUT if set
 int read_timeout_flag(const dfm_op* op, cudaStream_t st, const char* who);
 // bases above N_p = 8 (wide.cu).  pairs: the assembly's per-pair constants

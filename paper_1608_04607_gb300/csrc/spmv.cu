@@ -562,6 +562,10 @@ int launch(const dfm_op* op, const TX* x, const TX* x0, TX* y, int R, double alp
     // row, on tensor cores (spmv_mma.cu)
     if constexpr (std::is_same<TV, __nv_bfloat16>::value && std::is_same<TX, float>::value)
       if (K == 1 && !combo_ops && apply_mma_supported(op, R)) return apply_mma(op, x, x0, y, R, alpha, st);
+    // FP32 blocks and vectors where the tensor-core kernel is faster (both
+    // operands split, spmv_multi.cu)
+    if constexpr (std::is_same<TV, float>::value && std::is_same<TX, float>::value)
+      if (apply_multi_supported(op, K, R)) return apply_multi(op, combo_ops, K, coef, x, x0, y, R, alpha, st);
     if (R > kMaxStagedRhs) {  // several passes, each staging up to kMaxStagedRhs right-hand sides
       const int64_t stride = op->nrows * (int64_t)op->nb;
       for (int r0 = 0; r0 < R; r0 += kMaxStagedRhs) {
