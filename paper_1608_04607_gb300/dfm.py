@@ -586,6 +586,11 @@ class DFMSolve:
     def apply(mesh, Np, mu, rho0, tol=1e-8, **solve_kw):
         import torch
 
+        # the adjoint solve is preconditioned as the forward one: its polynomial
+        # then also runs on a low-precision (transposed) copy, and on none if
+        # the forward solve asked for none
+        adj_kw = dict(tol=tol, precond_precision=solve_kw.get("precond_precision", 0))
+
         def _grad_mu(per_tet):
             # a scalar (uniform) damping moves every tet's mu together
             if mu.dim() == 0:
@@ -612,11 +617,11 @@ class DFMSolve:
                     # one adjoint solve per distinct functional
                     grads, lams = [], []
                     for r in range(gsum.shape[0]):
-                        lam, dj, _ = op.adjoint(rho[r:r + 1], gsum[r], tol=tol)
+                        lam, dj, _ = op.adjoint(rho[r:r + 1], gsum[r], **adj_kw)
                         grads.append(dj[0])
                         lams.append(lam)
                     return _grad_mu(torch.stack(grads).sum(0)), torch.stack(lams)
-                lam, dj, _ = op.adjoint(rho, gsum.reshape(op.n_rows, op.nb), tol=tol)
+                lam, dj, _ = op.adjoint(rho, gsum.reshape(op.n_rows, op.nb), **adj_kw)
                 return _grad_mu(dj.sum(0)), lam.reshape(rho0.shape)
 
         return _Fn.apply(mu, rho0)

@@ -130,3 +130,42 @@ def test_autograd_function(D, problem):
     _, dj, _ = op.adjoint(r2, g, None, tol=1e-12)
     np.testing.assert_allclose(mu.grad.cpu().numpy(), dj[0].cpu().numpy(), rtol=1e-6,
                                atol=1e-9 * float(dj.abs().max()))
+
+
+@pytest.mark.parametrize("Np,R,n", [(0, 1, 2), (1, 3, 2), (2, 7, 2), (4, 8, 2), (5, 33, 1), (6, 2, 2), (7, 9, 2), (8, 1, 2)])
+def test_contraction_matches_blocks(D, Np, R, n):
+    """lambda^T (dB/dmu) rho per tet against the assembled first damping moment
+    (the same dB/dmu from another kernel): one to two columns of lanes, few
+    and many right-hand sides.  Both sums are FP32 over the same nodes: 1e-5 of
+    the largest entry, the entry tolerance of the blocks."""
+    import torch
+
+    m = kuhn_cube_mesh(n, jitter=0.2 if n > 1 else 0.0, seed=6)
+    mesh = D.Mesh(m.verts, m.tets, refl=0.9)
+    op, d1 = D.Operator(mesh, Np, mu=0.7), D.Operator(mesh, Np, mu=0.7, moment=1)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    rho = torch.randn((R, op.n_rows, op.nb), generator=g, device="cuda", dtype=torch.float64)
+    gvec = torch.randn((op.n_rows, op.nb), generator=g, device="cuda", dtype=torch.float64)
+    lam, dj, _ = op.adjoint(rho, gvec, tol=1e-8)
+    per_row = (d1.apply(rho) * lam).sum(-1)
+    tet = torch.from_numpy(mesh.recv().astype(np.int64) // 4).cuda()  # the tet a row receives from
+    want = torch.zeros((R, m.n_tets), dtype=torch.float64, device="cuda").index_add_(1, tet, per_row)
+    assert float((dj - want).abs().max()) <= 1e-5 * float(want.abs().max())
+
+
+def test_autograd_gradient_with_a_preconditioned_adjoint(D):
+    """precond_precision reaches the adjoint solve too; both solve to 1e-10, so
+    the gradients agree to that times the conditioning (below 100 here)."""
+    import torch
+
+    m = kuhn_cube_mesh(2, jitter=0.2, seed=6)
+    mesh = D.Mesh(m.verts, m.tets, refl=0.9)
+    rho0 = D.source(mesh, 4, [0, 5])
+    g = torch.randn(rho0.shape, generator=torch.Generator(device="cuda").manual_seed(1), device="cuda",
+                    dtype=torch.float64)
+    grads = []
+    for kw in ({}, {"precond_precision": D.FP8E4M3}):
+        mu = torch.full((m.n_tets,), 0.3, device="cuda", dtype=torch.float64, requires_grad=True)
+        (D.DFMSolve.apply(mesh, 4, mu, rho0, 1e-10, **kw) * g).sum().backward()
+        grads.append(mu.grad)
+    assert float((grads[0] - grads[1]).abs().max()) <= 1e-8 * float(grads[0].abs().max())
