@@ -157,7 +157,7 @@ hop_frag_kernel(const unsigned char* __restrict__ vals, const int32_t* __restric
   const int64_t x0_off = x_off + (int64_t)rpt * rgl * 4 * XR;
   const int64_t stage_bytes = x0_off + (int64_t)rgl * rpt * XR;
   const int64_t ntiles = (nrows + rpt - 1) / rpt;
-  const int64_t mine = ntiles > (int64_t)blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  const int mine = ntiles > (int64_t)blockIdx.x ? (int)((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   // one right-hand side: a source face row is only 2 NBP bytes, too small for
@@ -181,7 +181,7 @@ hop_frag_kernel(const unsigned char* __restrict__ vals, const int32_t* __restric
     // ---------------- producer ----------------
     const uint64_t pol_last = l2_policy_evict_last();
     const uint64_t pol_first = l2_policy_evict_first();
-    int64_t issued = 0;
+    int issued = 0;
     bool ok = true;
     // forward: the source tet of row R (recv[R] / 4), its 4 faces consecutive
     // rows; transposed: the receiving rows recv[4t + l'] of the row's own tet
@@ -198,8 +198,9 @@ hop_frag_kernel(const unsigned char* __restrict__ vals, const int32_t* __restric
       const int64_t R0 = tile_first_row(0);
       if (lane < rpt && R0 + lane < nrows) next_src = row_sources(R0 + lane);
     }
-    for (int64_t i = 0; i < mine && ok; ++i) {
-      const int s = (int)(i % stages);
+    int s = 0;        // stage of tile i and parity of its round
+    unsigned ph = 0;
+    for (int i = 0; i < mine && ok; ++i) {
       const int64_t R0 = tile_first_row(i);
       const int nr = (int)std::min<int64_t>(rpt, nrows - R0);
       const int4 src = next_src;
@@ -207,7 +208,7 @@ hop_frag_kernel(const unsigned char* __restrict__ vals, const int32_t* __restric
         const int64_t R1 = tile_first_row(i + 1);
         if (lane < rpt && R1 + lane < nrows) next_src = row_sources(R1 + lane);
       }
-      if (i >= stages) ok = mbar_wait_bounded(&empty[s], (unsigned)(((i / stages) - 1) & 1));
+      if (i >= stages) ok = mbar_wait_bounded(&empty[s], ph ^ 1u);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       unsigned char* st = stage0 + s * stage_bytes;
@@ -265,11 +266,15 @@ hop_frag_kernel(const unsigned char* __restrict__ vals, const int32_t* __restric
         }
       }
       issued = i + 1;
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     if (!ok && lane == 0) atomicOr(err, 1);
     // drain: every issued stage must have landed before the block's shared memory goes away
     if (lane == 0)
-      for (int64_t j = (issued > stages ? issued - stages : 0); j < issued; ++j)
+      for (int j = (issued > stages ? issued - stages : 0); j < issued; ++j)
         mbar_wait_bounded(&full[j % stages], (unsigned)((j / stages) & 1));
     return;
   }
@@ -277,9 +282,10 @@ hop_frag_kernel(const unsigned char* __restrict__ vals, const int32_t* __restric
   const int cgrp = (warp - 1) / kFragGroupWarps;
   const int cw = (warp - 1) % kFragGroupWarps;
   const int g8 = lane >> 2, t4 = lane & 3;
-  for (int64_t i = cgrp; i < mine; i += kFragGroups) {
-    const int s = (int)(i % stages);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (unsigned)((i / stages) & 1)));
+  int s = cgrp;  // stages are a multiple of the groups
+  unsigned ph = 0;
+  for (int i = cgrp; i < mine; i += kFragGroups) {
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], ph));
     if (!ok) {
       if (lane == 0) atomicOr(err, 1);
       break;
@@ -363,6 +369,10 @@ hop_frag_kernel(const unsigned char* __restrict__ vals, const int32_t* __restric
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
+    if ((s += kFragGroups) >= stages) {
+      s -= stages;
+      ph ^= 1u;
+    }
   }
 }
 

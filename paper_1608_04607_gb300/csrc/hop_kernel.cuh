@@ -22,7 +22,9 @@ namespace hopk {
 
 using namespace pipe;
 
-constexpr int kHopStages = 2;  // with 32-row tiles: 29.5 us per e4m3 hop (3 stages: 30.8, 4: 30.9)
+// Two stages with 32-row tiles (29.5 us per e4m3 hop at N_b = 15; 3 stages: 30.8, 4: 30.9);
+// a launch always has both, so a tile's stage and phase need no run-time division.
+constexpr int kHopStages = 2;
 // tile and stage geometry: launch_geometry.h (shared with the host-side check)
 using geom::kHopConsumerWarps;
 using geom::kHopMaxRhs;
@@ -170,7 +172,12 @@ hop_kernel(const unsigned char* __restrict__ vals, const int32_t* __restrict__ r
   const int64_t stage_bytes = (int64_t)RPT * ROW_BYTES + (int64_t)R * RPT * (XBLK + X0ROW);
   unsigned char* stage0 = smem_raw + 128 + ((kHopStages * RPT * 4 + 127) / 128) * 128;
   const int64_t ntiles = (nrows + RPT - 1) / RPT;
-  const int64_t mine = ntiles > (int64_t)blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  // tile counters: 32 bits for one right-hand side, where a tile's 64-bit
+  // arithmetic showed (48,000 tets, N_b = 15: 25.2 -> 23.5 us per hop); the
+  // launches of several measured 25% slower with them (8 right-hand sides, N_b =
+  // 21: 157 -> 198 us) and keep 64
+  using Count = std::conditional_t<(RC > 1), int64_t, int>;
+  const Count mine = ntiles > (int64_t)blockIdx.x ? (Count)((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -189,7 +196,7 @@ hop_kernel(const unsigned char* __restrict__ vals, const int32_t* __restrict__ r
     // ---------------- producer ----------------
     const uint64_t pol_last = l2_policy_evict_last();
     const uint64_t pol_first = l2_policy_evict_first();
-    int64_t issued = 0;
+    Count issued = 0;
     bool ok = true;
     // per tile row: the rows whose coefficients it gathers.  Forward: the
     // source tet of row R (recv[R] / 4), whose 4 faces are consecutive rows.
@@ -208,8 +215,8 @@ hop_kernel(const unsigned char* __restrict__ vals, const int32_t* __restrict__ r
       const int64_t R0 = tile_first_row(0);
       if (lane < RPT && R0 + lane < nrows) next_src = row_sources(R0 + lane);
     }
-    for (int64_t i = 0; i < mine && ok; ++i) {
-      const int s = (int)(i % stages);
+    for (Count i = 0; i < mine && ok; ++i) {
+      const int s = (int)(i % kHopStages);
       const int64_t R0 = tile_first_row(i);
       const int nr = (int)std::min<int64_t>(RPT, nrows - R0);
       const int4 src = next_src;
@@ -217,7 +224,7 @@ hop_kernel(const unsigned char* __restrict__ vals, const int32_t* __restrict__ r
         const int64_t R1 = tile_first_row(i + 1);
         if (lane < RPT && R1 + lane < nrows) next_src = row_sources(R1 + lane);
       }
-      if (i >= stages) ok = mbar_wait_bounded(&empty[s], (unsigned)(((i / stages) - 1) & 1));
+      if (i >= stages) ok = mbar_wait_bounded(&empty[s], (unsigned)(((i / kHopStages) - 1) & 1));
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       unsigned char* st = stage0 + s * stage_bytes;
@@ -262,7 +269,7 @@ hop_kernel(const unsigned char* __restrict__ vals, const int32_t* __restrict__ r
     if (!ok && lane == 0) atomicOr(err, 1);
     // drain: every issued stage must have landed before the block's shared memory goes away
     if (lane == 0)
-      for (int64_t j = (issued > stages ? issued - stages : 0); j < issued; ++j)
+      for (Count j = (issued > stages ? issued - stages : 0); j < issued; ++j)
         mbar_wait_bounded(&full[j % stages], (unsigned)((j / stages) & 1));
     return;
   }
@@ -270,9 +277,9 @@ hop_kernel(const unsigned char* __restrict__ vals, const int32_t* __restrict__ r
   const int ctid = threadIdx.x - 32;
   const int r0c = ctid / NBP;
   const int a = ctid - r0c * NBP;
-  for (int64_t i = 0; i < mine; ++i) {
-    const int s = (int)(i % stages);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (unsigned)((i / stages) & 1)));
+  for (Count i = 0; i < mine; ++i) {
+    const int s = (int)(i % kHopStages);
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (unsigned)((i / kHopStages) & 1)));
     if (!ok) {
       if (lane == 0) atomicOr(err, 1);
       break;

@@ -195,7 +195,7 @@ spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ 
   const int64_t stage_bytes = vals_bytes + (int64_t)R * rows_per_tile * xblk + ((x0_bytes + 15) / 16) * 16;
   unsigned char* stage0 = smem_raw + 128 + ((stages * rows_per_tile * 4 + 127) / 128) * 128;
   const int64_t ntiles = (nrows + rows_per_tile - 1) / rows_per_tile;
-  const int64_t mine = ntiles > (int64_t)blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  const int mine = ntiles > (int64_t)blockIdx.x ? (int)((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -210,7 +210,7 @@ spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ 
     // ---------------- producer ----------------
     // lane r handles tile row r (rows_per_tile <= 32); the row map of the next
     // tile is loaded one iteration ahead so its latency overlaps this tile's issue
-    int64_t issued = 0;
+    int issued = 0;
     bool ok = true;
     auto tile_rows = [&](int64_t i, int64_t* R0, int* nr) {
       const int64_t tile = blockIdx.x + i * (int64_t)gridDim.x;
@@ -230,8 +230,9 @@ spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ 
       tile_rows(0, &R0, &nr);
       if (lane < nr) next_src = recv[R0 + lane];
     }
-    for (int64_t i = 0; i < mine && ok; ++i) {
-      const int s = (int)(i % stages);
+    int s = 0;        // stage of tile i and parity of its round
+    unsigned ph = 0;
+    for (int i = 0; i < mine && ok; ++i) {
       int64_t R0;
       int nr;
       tile_rows(i, &R0, &nr);
@@ -242,7 +243,7 @@ spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ 
         tile_rows(i + 1, &R1, &n1);
         if (lane < n1) next_src = recv[R1 + lane];
       }
-      if (i >= stages) ok = mbar_wait_bounded(&empty[s], (unsigned)(((i / stages) - 1) & 1));
+      if (i >= stages) ok = mbar_wait_bounded(&empty[s], ph ^ 1u);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       unsigned char* st = stage0 + s * stage_bytes;
@@ -268,11 +269,15 @@ spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ 
           bulk_copy_g2s(st + vals_bytes + ((int64_t)rhs * rows_per_tile + lane) * xblk,
                         x + ((int64_t)rhs * nrows + 4 * (int64_t)(src >> 2)) * NB, (unsigned)xblk, &full[s]);
       issued = i + 1;
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     if (!ok && lane == 0) atomicOr(err, 1);
     // drain: every issued stage must have landed before the block's shared memory goes away
     if (lane == 0)
-      for (int64_t j = (issued > stages ? issued - stages : 0); j < issued; ++j)
+      for (int j = (issued > stages ? issued - stages : 0); j < issued; ++j)
         mbar_wait_bounded(&full[j % stages], (unsigned)((j / stages) & 1));
     return;
   }
@@ -281,9 +286,10 @@ spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ 
   constexpr bool kSplit = std::is_same<TX, double>::value && !std::is_same<TV, double>::value;
   const int ctid = threadIdx.x - 32;
   const int nthreads = 32 * kConsumerWarps;
-  for (int64_t i = 0; i < mine; ++i) {
-    const int s = (int)(i % stages);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (unsigned)((i / stages) & 1)));
+  int s = 0;
+  unsigned ph = 0;
+  for (int i = 0; i < mine; ++i) {
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], ph));
     if (!ok) {
       if (lane == 0) atomicOr(err, 1);
       break;
@@ -372,6 +378,10 @@ spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ 
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
+    if (++s == stages) {
+      s = 0;
+      ph ^= 1u;
+    }
   }
 }
 
@@ -399,7 +409,7 @@ spmv_t_tma_kernel(const TV* __restrict__ vals, int64_t row_stride, const int32_t
   const int64_t stage_bytes = rpt * row_bytes + xs_bytes;
   unsigned char* stage0 = smem_raw + 128;
   const int64_t ntiles = (nt + tets_per_tile - 1) / tets_per_tile;
-  const int64_t mine = ntiles > (int64_t)blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  const int mine = ntiles > (int64_t)blockIdx.x ? (int)((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -418,7 +428,7 @@ spmv_t_tma_kernel(const TV* __restrict__ vals, int64_t row_stride, const int32_t
   };
   if (warp == 0) {
     // ---------------- producer ----------------
-    int64_t issued = 0;
+    int issued = 0;
     bool ok = true;
     int32_t next_row = 0;
     TA next_x[NB];
@@ -434,8 +444,9 @@ spmv_t_tma_kernel(const TV* __restrict__ vals, int64_t row_stride, const int32_t
       }
     };
     if (mine > 0) fetch(0, &next_row, next_x);
-    for (int64_t i = 0; i < mine && ok; ++i) {
-      const int s = (int)(i % stages);
+    int s = 0;        // stage of tile i and parity of its round
+    unsigned ph = 0;
+    for (int i = 0; i < mine && ok; ++i) {
       int64_t T0;
       int ntt;
       tile_tets(i, &T0, &ntt);
@@ -444,7 +455,7 @@ spmv_t_tma_kernel(const TV* __restrict__ vals, int64_t row_stride, const int32_t
 #pragma unroll
       for (int a = 0; a < NB; ++a) xv[a] = next_x[a];
       if (i + 1 < mine) fetch(i + 1, &next_row, next_x);
-      if (i >= stages) ok = mbar_wait_bounded(&empty[s], (unsigned)(((i / stages) - 1) & 1));
+      if (i >= stages) ok = mbar_wait_bounded(&empty[s], ph ^ 1u);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       unsigned char* st = stage0 + s * stage_bytes;
@@ -459,19 +470,24 @@ spmv_t_tma_kernel(const TV* __restrict__ vals, int64_t row_stride, const int32_t
       if (lane == 0) mbar_arrive_expect_tx(&full[s], (unsigned)(nr * row_bytes));
       if (lane < nr) bulk_copy_g2s(st + lane * row_bytes, vals + (int64_t)row * row_stride, (unsigned)row_bytes, &full[s]);
       issued = i + 1;
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     if (!ok && lane == 0) atomicOr(err, 1);
     if (lane == 0)
-      for (int64_t j = (issued > stages ? issued - stages : 0); j < issued; ++j)
+      for (int j = (issued > stages ? issued - stages : 0); j < issued; ++j)
         mbar_wait_bounded(&full[j % stages], (unsigned)((j / stages) & 1));
     return;
   }
   // ---------------- consumers ----------------
   const int ctid = threadIdx.x - 32;
   const int nthreads = 32 * kConsumerWarps;
-  for (int64_t i = 0; i < mine; ++i) {
-    const int s = (int)(i % stages);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (unsigned)((i / stages) & 1)));
+  int s = 0;
+  unsigned ph = 0;
+  for (int i = 0; i < mine; ++i) {
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], ph));
     if (!ok) {
       if (lane == 0) atomicOr(err, 1);
       break;
@@ -503,6 +519,10 @@ spmv_t_tma_kernel(const TV* __restrict__ vals, int64_t row_stride, const int32_t
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
+    if (++s == stages) {
+      s = 0;
+      ph ^= 1u;
+    }
   }
 }
 

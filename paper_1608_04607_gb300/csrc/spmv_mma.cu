@@ -87,7 +87,7 @@ spmv_mma_kernel(const __nv_bfloat16* __restrict__ vals, int64_t row_stride, cons
   const int64_t stage_bytes = x_off + (int64_t)rpt * R * XB;
   const int ng = (R + 7) / 8;
   const int64_t ntiles = (nrows + rpt - 1) / rpt;
-  const int64_t mine = ntiles > (int64_t)blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  const int mine = ntiles > (int64_t)blockIdx.x ? (int)((ntiles - 1 - blockIdx.x) / gridDim.x) + 1 : 0;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -106,15 +106,16 @@ spmv_mma_kernel(const __nv_bfloat16* __restrict__ vals, int64_t row_stride, cons
     // ---------------- producer ----------------
     const uint64_t pol_last = l2_policy_evict_last();
     const uint64_t pol_first = l2_policy_evict_first();
-    int64_t issued = 0;
+    int issued = 0;
     bool ok = true;
     int32_t next_src = 0;
     if (mine > 0) {
       const int64_t R0 = tile_first_row(0);
       if (lane < rpt && R0 + lane < nrows) next_src = recv[R0 + lane];
     }
-    for (int64_t i = 0; i < mine && ok; ++i) {
-      const int s = (int)(i % stages);
+    int s = 0;        // stage of tile i and parity of its round
+    unsigned ph = 0;
+    for (int i = 0; i < mine && ok; ++i) {
       const int64_t R0 = tile_first_row(i);
       const int nr = (int)std::min<int64_t>(rpt, nrows - R0);
       const int32_t src = next_src;
@@ -122,7 +123,7 @@ spmv_mma_kernel(const __nv_bfloat16* __restrict__ vals, int64_t row_stride, cons
         const int64_t R1 = tile_first_row(i + 1);
         if (lane < rpt && R1 + lane < nrows) next_src = recv[R1 + lane];
       }
-      if (i >= stages) ok = mbar_wait_bounded(&empty[s], (unsigned)(((i / stages) - 1) & 1));
+      if (i >= stages) ok = mbar_wait_bounded(&empty[s], ph ^ 1u);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       unsigned char* st = stage0 + s * stage_bytes;
@@ -144,10 +145,14 @@ spmv_mma_kernel(const __nv_bfloat16* __restrict__ vals, int64_t row_stride, cons
                         &full[s]);
       }
       issued = i + 1;
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
     if (!ok && lane == 0) atomicOr(err, 1);
     if (lane == 0)
-      for (int64_t j = (issued > stages ? issued - stages : 0); j < issued; ++j)
+      for (int j = (issued > stages ? issued - stages : 0); j < issued; ++j)
         mbar_wait_bounded(&full[j % stages], (unsigned)((j / stages) & 1));
     return;
   }
@@ -155,9 +160,10 @@ spmv_mma_kernel(const __nv_bfloat16* __restrict__ vals, int64_t row_stride, cons
   const int cgrp = (warp - 1) / kGroupWarps;
   const int cw = (warp - 1) % kGroupWarps;
   const int g8 = lane >> 2, t4 = lane & 3;
-  for (int64_t i = cgrp; i < mine; i += kGroups) {
-    const int s = (int)(i % stages);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], (unsigned)((i / stages) & 1)));
+  int s = cgrp;  // stages are a multiple of the groups
+  unsigned ph = 0;
+  for (int i = cgrp; i < mine; i += kGroups) {
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&full[s], ph));
     if (!ok) {
       if (lane == 0) atomicOr(err, 1);
       break;
@@ -228,6 +234,10 @@ spmv_mma_kernel(const __nv_bfloat16* __restrict__ vals, int64_t row_stride, cons
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[s]);
+    if ((s += kGroups) >= stages) {
+      s -= stages;
+      ph ^= 1u;
+    }
   }
 }
 
