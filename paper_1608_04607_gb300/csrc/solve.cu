@@ -398,6 +398,212 @@ inline int precond_hops(const Ctx& c, const Hop& hp, int R, int d, const float* 
 
 #include "block_gmres.cuh"
 
+// ---------------------------------------------------------------------------
+// Neumann series of a small FP64 operator in one launch.  The series needs one
+// application and one norm per term; on a small mesh these take a few
+// microseconds each and the launches, the norm's copy to the host and the wait
+// for it ten times as long.  Here co-resident blocks (cooperative launch) keep
+// their operator rows in shared memory for the whole solve, exchange the iterate
+// through L2 and meet at a grid barrier per term, where each block sums every
+// block's share of the norms and decides alike.  The arithmetic of a term is
+// that of spmv.cu's row_times_x, in the same order.  Barrier waits are bounded.
+// Measured: 6 tets, 6 functions (276 terms) in 1.07 ms against 8.8 ms; 1,296
+// tets, 15 functions (2,958 terms) in 49 against 129 ms.
+// ---------------------------------------------------------------------------
+struct NeumannState {
+  unsigned long long bar;  // arrivals at the grid barrier
+  int iters, status;       // terms taken; DFM_OK or an error
+};
+constexpr int kNeumannThreads = 256;
+constexpr long long kNeumannPolls = 1ll << 22;
+
+// sums of both values over the block, valid in thread 0
+__device__ __forceinline__ void block_sum2(double& a, double& b, double2* sh) {
+  a = warp_sum(a);
+  b = warp_sum(b);
+  __syncthreads();  // the previous sums are read
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = make_double2(a, b);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a = b = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      a += sh[w].x;
+      b += sh[w].y;
+    }
+  }
+}
+
+// ONE: a single block, the iterate in its shared memory as well
+template <bool ONE>
+__global__ void __launch_bounds__(kNeumannThreads)
+neumann_kernel(const double* __restrict__ vals, int64_t row_stride, const int32_t* __restrict__ recv, int nrows, int nb,
+               int rows_pb, const double* __restrict__ b, double* xa, double* xb, double tol, int max_iter,
+               double* partial, NeumannState* st, int* __restrict__ err) {
+  extern __shared__ __align__(16) double nsm_buf[];
+  __shared__ double2 sh[kNeumannThreads / 32];
+  __shared__ double2 tot;
+  __shared__ int s_ok;
+  const int r0 = blockIdx.x * rows_pb, nr = min(rows_pb, nrows - r0);
+  const int rs = (int)row_stride, nb2 = nb * nb, nx = 3 * nb;
+  double* B = nsm_buf;               // [rows_pb][row_stride]
+  double* xs = B + rows_pb * rs;     // [rows_pb][3 nb] the rows' source coefficients
+  int* src_at = reinterpret_cast<int*>(xs + rows_pb * nx);  // where they come from
+  double* sx = reinterpret_cast<double*>(src_at + (rows_pb * nx + 1) / 2 * 2);  // ONE: two iterates
+  for (int i = threadIdx.x; i < nr * rs; i += blockDim.x) B[i] = vals[(int64_t)r0 * rs + i];
+  for (int i = threadIdx.x; i < nr * nx; i += blockDim.x) {
+    const int r = i / nx, e = i - r * nx, k = e / nb;
+    const int32_t src = recv[r0 + r];
+    src_at[i] = (4 * (src >> 2) + k + (k >= (src & 3) ? 1 : 0)) * nb + e - k * nb;
+  }
+  const int n = nr * nb;
+  double *cur = xa, *nxt = xb;
+  if constexpr (ONE) {
+    cur = sx;
+    nxt = sx + n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) cur[i] = xa[i];
+  }
+  __syncthreads();
+  auto get = [](const double* p) { return ONE ? *p : __ldcg(p); };
+  const int own = ONE ? 0 : r0 * nb;  // this block's part of the iterate
+  int it = 0, status = DFM_OK;
+  while (true) {
+    for (int i = threadIdx.x; i < nr * nx; i += blockDim.x) xs[i] = get(cur + src_at[i]);
+    __syncthreads();
+    double d2 = 0.0, a2 = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+      const int r = i / nb, a = i - r * nb;
+      const double* br = B + r * rs + a * nb;
+      const double* xr = xs + r * nx;
+      double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0;
+      for (int c = 0; c < nb; ++c) {
+        acc0 = fma(br[c], xr[c], acc0);
+        acc1 = fma(br[nb2 + c], xr[nb + c], acc1);
+        acc2 = fma(br[2 * nb2 + c], xr[2 * nb + c], acc2);
+      }
+      const double v = b[r0 * nb + i] + ((acc0 + acc1) + acc2);
+      const double d = v - get(cur + own + i);
+      if (ONE) nxt[i] = v;
+      else __stcg(nxt + own + i, v);
+      d2 = fma(d, d, d2);
+      a2 = fma(v, v, a2);
+    }
+    ++it;
+    block_sum2(d2, a2, sh);
+    if constexpr (ONE) {
+      if (threadIdx.x == 0) tot = make_double2(d2, a2);
+      __syncthreads();
+    } else {
+      double* slot = partial + (it & 1) * 2 * gridDim.x;  // the other terms' slots may still be read
+      if (threadIdx.x == 0) {
+        __stcg(slot + 2 * blockIdx.x, d2);
+        __stcg(slot + 2 * blockIdx.x + 1, a2);
+        __threadfence();
+        atomicAdd(&st->bar, 1ull);
+        const unsigned long long want = (unsigned long long)it * gridDim.x;
+        bool ok = false;
+        for (long long p = 0; p < kNeumannPolls && !ok; ++p)
+          ok = *reinterpret_cast<volatile unsigned long long*>(&st->bar) >= want;
+        __threadfence();
+        s_ok = ok;
+      }
+      __syncthreads();
+      if (!s_ok) {  // a block never arrived
+        if (threadIdx.x == 0) atomicOr(err, 1);
+        status = DFM_ERR_TIMEOUT;
+        break;
+      }
+      if (threadIdx.x < 32) {
+        double t1 = 0.0, t2 = 0.0;
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) {
+          t1 += __ldcg(slot + 2 * i);
+          t2 += __ldcg(slot + 2 * i + 1);
+        }
+        t1 = warp_sum(t1);
+        t2 = warp_sum(t2);
+        if (threadIdx.x == 0) tot = make_double2(t1, t2);
+      }
+      __syncthreads();
+    }
+    const double dd = tot.x, aa = tot.y;
+    double* tmp = cur;
+    cur = nxt;
+    nxt = tmp;
+    if (!(dd == dd) || isinf(dd)) {
+      status = DFM_ERR_NONFINITE;
+      break;
+    }
+    if (sqrt(dd) <= tol * sqrt(aa)) break;
+    if (it >= max_iter) {
+      status = DFM_ERR_NOT_CONVERGED;
+      break;
+    }
+  }
+  if (cur != xa)  // leave the last iterate in xa (this block's own rows)
+    for (int i = threadIdx.x; i < n; i += blockDim.x) xa[r0 * nb + i] = get(cur + own + i);
+  if (threadIdx.x == 0 && blockIdx.x == 0) {
+    st->iters = it;
+    st->status = status;
+  }
+}
+
+struct NeumannGeo {
+  int grid = 0, rows_pb = 0, threads = 0;
+  size_t smem = 0;
+};
+
+// Blocks and rows per block, or grid = 0 where the operator does not fit the
+// shared memory of one block per SM (30 MB in all), or has no FP64 blocks of
+// the narrow bases, or reflected parts.  A block takes at least 4,000 FP64
+// multiply-adds per term (about 1 us on its SM's two lanes, what a barrier
+// costs) before the rows are spread over more of them.
+inline NeumannGeo neumann_geometry(const Ctx& c) {
+  const dfm_op* op = c.op;
+  NeumannGeo g;
+  if (op->precision != DFM_F64 || op->rop || c.combo || c.trans || op->ns != 1 || !narrow_nb(op->nb) ||
+      op->nrows > (1 << 20))
+    return g;
+  const int64_t per_row = 8 * (op->row_stride + 3 * op->nb) + 4 * 3 * op->nb, most = 220 * 1024;
+  const int64_t fit = most / per_row;
+  if (fit < 1 || (op->nrows + fit - 1) / fit > c.nsm) return g;
+  const int64_t macs = op->nrows * 3 * op->nb * op->nb;
+  int64_t grid = std::max((op->nrows + fit - 1) / fit, std::min<int64_t>(c.nsm, macs / 4000));
+  grid = std::max<int64_t>(1, std::min(grid, op->nrows));
+  g.rows_pb = (int)((op->nrows + grid - 1) / grid);
+  g.grid = (int)((op->nrows + g.rows_pb - 1) / g.rows_pb);
+  g.smem = (size_t)(g.rows_pb * per_row) + 8;
+  if (g.grid == 1) g.smem += 16 * (size_t)(g.rows_pb * op->nb);
+  if (g.smem > 226 * 1024) g.grid = 0;
+  // no more warps than elements: an idle warp's share of the sums costs FP64 issue too
+  g.threads = std::min(kNeumannThreads, (g.rows_pb * op->nb + 31) / 32 * 32);
+  return g;
+}
+
+// x <- b + B x until |x_new - x| <= tol |x_new| (x: initial guess and result);
+// work: n doubles, partial: 4 nsm doubles and the state.  Returns DFM_OK, the
+// series' status in *status, or an error of the launch.
+inline int neumann_small(const Ctx& c, const NeumannGeo& g, const double* b, double* x, double* work, double* partial,
+                         double tol, int max_iter, int* iters, int* status) {
+  NeumannState* st = reinterpret_cast<NeumannState*>(partial + 4 * (int64_t)g.grid);
+  DFM_CUDA_CHECK(cudaMemsetAsync(st, 0, sizeof(NeumannState), c.st));
+  auto* kernel = g.grid == 1 ? neumann_kernel<true> : neumann_kernel<false>;
+  DFM_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+  const double* vals = reinterpret_cast<const double*>(c.op->vals);
+  int64_t row_stride = c.op->row_stride;
+  const int32_t* recv = c.op->recv ? c.op->recv : c.op->mesh->recv;
+  int nrows = (int)c.op->nrows, nb = c.op->nb, rows_pb = g.rows_pb;
+  int* err = c.op->dev_err;
+  void* args[] = {&vals, &row_stride, &recv, &nrows, &nb, &rows_pb, &b, &x, &work, &tol, &max_iter, &partial, &st, &err};
+  DFM_CUDA_CHECK(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3((unsigned)g.grid),
+                                             dim3((unsigned)g.threads), args, g.smem, c.st));
+  DFM_LAUNCHED();
+  NeumannState h;
+  DFM_CUDA_CHECK(cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, c.st));
+  DFM_CUDA_CHECK(cudaStreamSynchronize(c.st));
+  *iters = h.iters;
+  *status = h.status;
+  return DFM_OK;
+}
+
 // Two-level correction of the flexible preconditioner (dfm_solve_opts.coarse;
 // not in the paper, the solver acceleration its slow modes call for): the
 // slowest mode of I - B at small loss is the isotropic density, so a coarse
@@ -1243,8 +1449,17 @@ int solve_impl(const dfm_op* op, const dfm_op* const* combo, int K, const double
     int rs = DFM_OK;
     if (method == DFM_SOLVE_NEUMANN) {
       // x <- rho0 + B x until |x_new - x| <= tol |x_new|
+      const NeumannGeo ng = neumann_geometry(c);
+      if (ng.grid) {
+        int ns = DFM_OK;
+        const int r2 = neumann_small(c, ng, b, x, xold, part64, opts->tol, max_iter, &iters, &ns);
+        if (r2) return r2;
+        if (ns == DFM_ERR_NONFINITE) rs = set_error(ns, "dfm_solve: non-finite Neumann iterate");
+        if (ns == DFM_ERR_NOT_CONVERGED) rs = set_error(ns, "dfm_solve: Neumann series reached max_iter");
+        // (a barrier that timed out is reported from the operator's flag below)
+      }
       std::vector<double> ph(2 * kRedBlocks);
-      while (true) {
+      while (!ng.grid) {
         DFM_CUDA_CHECK(cudaMemcpyAsync(xold, x, sizeof(double) * n, cudaMemcpyDeviceToDevice, c.st));
         rs = ctx_apply(c, xold, b, x, 1, 1.0, DFM_F64);
         if (rs) return rs;

@@ -27,6 +27,7 @@
 #include "interior_rule.cuh"
 #include "node.cuh"
 #include "p1_basis.h"
+#include "tma_pipe.cuh"
 #include "zernike_wide.h"
 
 namespace dfm {
@@ -336,6 +337,217 @@ spmv_wide_kernel(const float* __restrict__ vals, int64_t row_stride, const int32
 }
 
 // ---------------------------------------------------------------------------
+// The same for FP32 vectors with the blocks streamed by bulk copies (TMA): a
+// chunk is the three blocks' rows of kWAc consecutive test indices (one
+// contiguous piece of each block, its start rounded down to 16 bytes), and a
+// block of the grid walks a contiguous range of all chunks with a ring of chunk
+// stages and two slots for the operator row's source coefficients.  Two groups
+// of eight warps take alternate chunks (the stages are even in number), warp w of
+// a group test indices w and w + 8: a chunk's time is the latency of one warp's
+// wait, sums and shuffles (0.6 us), and with one group and eight indices per
+// chunk that was all of it (254 us).  A staged chunk serves every right-hand
+// side of the launch.  The sums are those of spmv_wide_kernel (lane-strided,
+// then shuffled).  Waits are bounded; a time-out sets the operator's flag.
+// Measured (768 tets, N_b = 153): 161 us (79% of the copy bandwidth) against 254
+// us for the kernel above, whose two block barriers per row left it at half.
+// ---------------------------------------------------------------------------
+constexpr int kWAc = 16;       // test indices per chunk (two per consumer warp)
+constexpr int kWWarps = 8;     // consumer warps of a group
+constexpr int kWGroups = 2;
+constexpr int kWMaxStages = 32;
+constexpr int kWMaxRhs = 8;    // right-hand sides per launch
+constexpr int kWHead = 1024;   // barriers
+static_assert((2 * kWMaxStages + 4) * 8 <= kWHead, "barriers");
+
+__global__ void __launch_bounds__(32 * (kWGroups * kWWarps + 1), 1)
+spmv_wide_tma_kernel(const float* __restrict__ vals, int64_t row_stride, const int32_t* __restrict__ recv, int64_t nrows,
+                     int nb, const float* __restrict__ x, const float* x0, float* y, int R, float alpha, int cpr,
+                     int stages, int* __restrict__ err) {
+  using namespace pipe;
+  extern __shared__ __align__(16) unsigned char spmv_wsm[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(spmv_wsm);
+  uint64_t* empty = full + kWMaxStages;
+  uint64_t* xfull = empty + kWMaxStages;
+  uint64_t* xempty = xfull + 2;
+  const int piece = kWAc * nb + 4;  // floats of one block's piece (a multiple of 4) with room for the rounding
+  float* stage0 = reinterpret_cast<float*>(spmv_wsm + kWHead);
+  float* slot0 = stage0 + (int64_t)stages * 3 * piece;
+  const int slot_f = R * 4 * nb;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], kWWarps);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&xfull[s], 1);
+      mbar_init(&xempty[s], kWGroups * kWWarps);
+    }
+    mbar_init_fence();
+  }
+  __syncthreads();
+  const int64_t chunks = nrows * cpr;
+  const int64_t per = (chunks + gridDim.x - 1) / gridDim.x;
+  const int64_t c0 = (int64_t)blockIdx.x * per, c1 = min(chunks, c0 + per);
+  const int64_t row0 = c0 / cpr;
+  const int a_first = (int)(c0 - row0 * cpr) * kWAc;
+  const int64_t nb2 = (int64_t)nb * nb;
+  const int n = c1 > c0 ? (int)(c1 - c0) : 0;
+  int s = 0;
+  unsigned ph = 0;
+  int64_t row = row0;
+  int a0 = a_first, rl = 0;  // rl: rows started by this block
+  bool ok = true;
+  if (warp == 0) {
+    // ---------------- producer ----------------
+    const uint64_t pol = l2_policy_evict_first();
+    int32_t next = n > 0 ? recv[row0] : 0;
+    int issued = 0;
+    for (int i = 0; i < n; ++i) {
+      const bool fresh = i == 0 || a0 == 0;
+      if (fresh) {
+        const int64_t t = next >> 2;
+        if (row + 1 < nrows) next = recv[row + 1];
+        const int xs = rl & 1;
+        if (rl >= 2) ok = mbar_wait_bounded(&xempty[xs], (unsigned)((rl >> 1) - 1) & 1u);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (lane == 0) mbar_arrive_expect_tx(&xfull[xs], (unsigned)slot_f * 4u);
+        __syncwarp();
+        if (lane < R)
+          bulk_copy_g2s(slot0 + xs * slot_f + lane * 4 * nb, x + (lane * nrows + 4 * t) * nb, 16u * nb, &xfull[xs]);
+        ++rl;
+      }
+      if (i >= stages) ok = mbar_wait_bounded(&empty[s], ph ^ 1u);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const int na = min(kWAc, nb - a0);
+      // floats of each piece: from the element rounded down to a multiple of 4
+      // to the end rounded up (the last piece ends within the row's padded stride)
+      const int64_t e0 = lane * nb2 + (int64_t)a0 * nb;
+      const int64_t lo = e0 & ~int64_t(3), hi = (e0 + na * nb + 3) & ~int64_t(3);
+      const unsigned bytes = lane < 3 ? (unsigned)(hi - lo) * 4u : 0u;
+      const unsigned sum = bytes + __shfl_down_sync(0xffffffffu, bytes, 1) + __shfl_down_sync(0xffffffffu, bytes, 2);
+      if (lane == 0) mbar_arrive_expect_tx(&full[s], sum);
+      __syncwarp();
+      if (lane < 3)
+        bulk_copy_g2s_hint(stage0 + ((int64_t)s * 3 + lane) * piece, vals + row * row_stride + lo, bytes, &full[s], pol);
+      issued = i + 1;
+      a0 += kWAc;
+      if (a0 >= nb) {
+        a0 = 0;
+        ++row;
+      }
+      if (++s == stages) {
+        s = 0;
+        ph ^= 1u;
+      }
+    }
+    if (!ok && lane == 0) atomicOr(err, 1);
+    // drain: every issued copy must have landed before the block's shared memory goes away
+    if (lane == 0) {
+      for (int i = issued > stages ? issued - stages : 0; i < issued; ++i)
+        mbar_wait_bounded(&full[i % stages], (unsigned)(i / stages) & 1u);
+      for (int i = rl > 2 ? rl - 2 : 0; i < rl; ++i) mbar_wait_bounded(&xfull[i & 1], (unsigned)(i >> 1) & 1u);
+    }
+    return;
+  }
+  // ---------------- consumers ----------------
+  const int w = (warp - 1) % kWWarps, grp = (warp - 1) / kWWarps;
+  int32_t e = 0, next = n > 0 ? recv[row0] : 0;
+  // x0 of this warp's outputs in a whole row, lane c + 16 h holding test index
+  // 16 c + 8 h + w (at most 16 chunks), one row ahead: loaded chunk by chunk, its
+  // latency would be the chunk's time
+  const int a_lane = kWAc * (lane & 15) + kWWarps * (lane >> 4) + w;
+  float base[kWMaxRhs], base_next[kWMaxRhs];
+  auto load_base = [&](int64_t rw) {
+#pragma unroll
+    for (int r = 0; r < kWMaxRhs; ++r)
+      base_next[r] = x0 && r < R && rw < nrows && a_lane < nb ? x0[(r * nrows + rw) * nb + a_lane] : 0.f;
+  };
+  if (n > 0) load_base(row0);
+  for (int i = 0; i < n; ++i) {
+    const int xs = (rl - 1) & 1;
+    int slot = xs;
+    if (i == 0 || a0 == 0) {
+      e = next & 3;
+      if (row + 1 < nrows) next = recv[row + 1];
+#pragma unroll
+      for (int r = 0; r < kWMaxRhs; ++r) base[r] = base_next[r];
+      load_base(row + 1);
+      slot = rl & 1;
+      ok = mbar_wait_bounded(&xfull[slot], (unsigned)(rl >> 1) & 1u);
+      ++rl;
+    }
+    const bool mine = (i & (kWGroups - 1)) == grp;
+    if (mine) ok = ok && mbar_wait_bounded(&full[s], ph);
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) {
+      if (lane == 0) atomicOr(err, 1);
+      break;
+    }
+    if (mine) {
+      const int a = a0 + w;
+      if (a < nb) {
+        const bool two = a + kWWarps < nb;
+        float bv[2][3][8];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const int64_t e0 = k * nb2 + (int64_t)a0 * nb;
+          const float* bp = stage0 + ((int64_t)s * 3 + k) * piece + (int)(e0 & 3) + w * nb;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {  // nb <= 256
+            const int j = lane + 32 * u;
+            bv[0][k][u] = j < nb ? bp[j] : 0.f;
+            bv[1][k][u] = two && j < nb ? bp[kWWarps * nb + j] : 0.f;
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < kWMaxRhs; ++r) {
+          if (r >= R) break;
+          const float* xr = slot0 + slot * slot_f + r * 4 * nb;
+          float acc[2] = {0.f, 0.f};
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            const float* xk = xr + (k + (k >= e ? 1 : 0)) * nb;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+              const int j = lane + 32 * u;
+              if (j < nb) {
+                const float xv = xk[j];
+                acc[0] = fmaf(bv[0][k][u], xv, acc[0]);
+                acc[1] = fmaf(bv[1][k][u], xv, acc[1]);
+              }
+            }
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) {
+            acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+            acc[1] += __shfl_xor_sync(0xffffffffu, acc[1], o);
+          }
+          if ((lane & 15) == a0 / kWAc && a_lane < nb)
+            y[(r * nrows + row) * nb + a_lane] = base[r] + alpha * (lane < 16 ? acc[0] : acc[1]);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s]);
+    }
+    a0 += kWAc;
+    if (a0 >= nb || i + 1 == n) {  // last chunk of this row here
+      if (lane == 0) mbar_arrive(&xempty[slot]);
+      if (a0 >= nb) {
+        a0 = 0;
+        ++row;
+      }
+    }
+    if (++s == stages) {
+      s = 0;
+      ph ^= 1u;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Directed boundary source (Eq. RhoNeumann), one thread per source: the
 // coefficients N_nm Z_n^m(p_d) sqrt|T| of the unit-mass delta at p_d.
 // ---------------------------------------------------------------------------
@@ -580,7 +792,35 @@ int apply_wide_t(const dfm_op* op, const TX* x, const TX* x0, TX* y, int R, doub
   return DFM_OK;
 }
 
+// FP32 vectors of the bases above N_p = 8, kWMaxRhs right-hand sides per launch
+int apply_wide_tma(const dfm_op* op, const float* x, const float* x0, float* y, int R, float alpha, cudaStream_t st) {
+  const int32_t* recv = op->recv ? op->recv : op->mesh->recv;
+  const int nb = op->nb, cpr = (nb + kWAc - 1) / kWAc;
+  const int64_t stride = op->nrows * (int64_t)nb;
+  for (int r0 = 0; r0 < R; r0 += kWMaxRhs) {
+    const int Rl = std::min(kWMaxRhs, R - r0);
+    const int64_t stage = 3 * (int64_t)(kWAc * nb + 4) * 4, slots = 2 * (int64_t)Rl * 4 * nb * 4;
+    const int stages = (int)std::min<int64_t>(kWMaxStages, (226 * 1024 - kWHead - slots) / stage) & ~1;
+    const size_t smem = kWHead + (size_t)(stages * stage + slots);
+    const int64_t grid = std::min<int64_t>(op->nrows * cpr, device_sms());
+    DFM_CUDA_CHECK(cudaFuncSetAttribute(spmv_wide_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    {
+      ::dfm::KernelTimer timer_(DFM_KERNEL_SPMV, st);
+      spmv_wide_tma_kernel<<<(unsigned)grid, 32 * (kWGroups * kWWarps + 1), smem, st>>>(
+          reinterpret_cast<const float*>(op->vals), op->row_stride, recv, op->nrows, nb, x + r0 * stride,
+          x0 ? x0 + r0 * stride : nullptr, y + r0 * stride, Rl, alpha, cpr, stages, op->dev_err);
+    }
+    DFM_LAUNCHED();
+    DFM_CUDA_CHECK(cudaGetLastError());
+  }
+  return DFM_OK;
+}
+
 int apply_wide(const dfm_op* op, const float* x, const float* x0, float* y, int R, double alpha, cudaStream_t st) {
+  // the streamed kernel from 55 functions on (below, the linear spatial basis'
+  // small blocks fill neither its chunks nor its lanes)
+  if (op->precision == DFM_F32 && op->nb >= 55 && op->nb <= 256)
+    return apply_wide_tma(op, x, x0, y, R, (float)alpha, st);
   return apply_wide_t<float>(op, x, x0, y, R, alpha, st);
 }
 
