@@ -27,7 +27,9 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
+#include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "row_node.cuh"

@@ -30,6 +30,8 @@
 #include "tma_pipe.cuh"
 #include "zernike_wide.h"
 
+#include "assemble_wide_mma.cuh"
+
 namespace dfm {
 namespace {
 
@@ -727,6 +729,9 @@ int launch_assemble_wide(int Np, const void* pairs, int64_t npairs, const double
   if (q < 1 || q > kMaxQ) return set_error(DFM_ERR_ARG, "dfm_assemble: quad_order must be in 1..32");
   if (npairs > 0x7fffffff) return set_error(DFM_ERR_ARG, "dfm_assemble: too many face pairs");
   if (npairs == 0) return DFM_OK;
+  if (Np >= kWideMmaMinNp)
+    return launch_assemble_wide_mma(Np, reinterpret_cast<const PairConst*>(pairs), npairs, glx, glw, q, cos_max, vals,
+                                    row_stride, nodes, moment, st);
   const geom::WideAsm G = geom::wide_asm_geometry(nbasis(Np));
   if (G.smem > 200 * 1024 || G.threads > 256)
     return set_error(DFM_ERR_UNSUPPORTED, "dfm_assemble: wide assembly tile does not fit a block");

@@ -206,3 +206,20 @@ def test_wide_interior_density_matches_oracle(D, oracle_mod):
     for t in tets[:2]:
         go, _ = oracle_mod.interior_g(m.verts, m.tets, t, cen[t], mu, 16, nq=32)
         assert np.abs(gf[4 * t:4 * t + 4] - go).max() <= 1e-11 * np.abs(go).max()
+
+
+@pytest.mark.parametrize("Np", range(9, 21))
+@pytest.mark.parametrize("quad_order,deg,mu,moment", [(1, 180.0, 0.0, 0), (7, 10.0, 0.4, 0), (32, 60.0, 40.0, 0),
+                                                      (13, 60.0, 0.3, 2)])
+def test_wide_blocks_contain_the_narrow_ones(D, cube2, Np, quad_order, deg, mu, moment):
+    """The basis is hierarchical, so under one explicit rule the first 45 x 45
+    entries of every block are the N_p = 8 block: compared with the FP64 operator,
+    from one node per patch to 1,024, on every order's tiling of the block.  The
+    node counts agree; entries to the FP32 entry tolerance of the block."""
+    mesh = D.Mesh(cube2.verts, cube2.tets, refl=0.8)
+    kw = dict(mu=mu, quad_order=quad_order, max_patch_deg=deg, moment=moment)
+    a, b = D.Operator(mesh, Np, **kw), D.Operator(mesh, 8, precision=D.F64, **kw)
+    assert D.op_nodes(a) == D.op_nodes(b)
+    full, y = a.blocks().double(), b.blocks()
+    err = (full[:, :, :45, :45] - y).abs().amax((2, 3)) / full.abs().amax((2, 3))
+    assert float(err.max()) <= 1e-5
