@@ -107,6 +107,17 @@ __device__ __forceinline__ void mma_f16(float d[4], const uint32_t a[4], uint32_
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// What the tensor cores' rounding towards zero takes off a pass's sum on average,
+// given back when the block is scaled.  hi hi runs over two MMAs, the first at
+// half the sum: 1.5 truncations of half a unit of 2^-23 / mantissa each, 1 / mantissa
+// being 0.72 on average: 6.4e-8.  Without it every entry is 7e-8 too small, and
+// solves at little damping magnify a loss common to all entries (gradients of
+// 384 tets at N_p = 6: 4.5e-6 off without it, 1.5e-6 with it, 2.8e-6 for FP32 sums in
+// sequence).  Where the three products have chains of their own, Z_0 = 1 makes hi hi
+// of column 0 exact, and nothing is given back there.
+constexpr float kTruncated = 6.4e-8f;
+__device__ __forceinline__ float scale_sum(float sum, float s) { return fmaf(sum, s, sum * s * kTruncated); }
+
 // acc += inv * (staged Z(p'))^T (staged Z(p)) over the 32 nodes of a pass.
 // ldmatrix.trans of the node-major rows gives both operands: the A fragment
 // of (m-tile, 16 nodes) from four 8 x 8 pieces, and the B fragments of both
@@ -266,7 +277,7 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
             for (int e = 0; e < 2; ++e) {
               const int b = 8 * nt + 2 * t4 + e;
               if (b >= NB) continue;
-              const float v = acc[nt][mt][2 * h + e] * s;
+              const float v = MT == 1 && b == 0 ? acc[nt][mt][2 * h + e] * s : scale_sum(acc[nt][mt][2 * h + e], s);
               if constexpr (std::is_same<TO, __nv_bfloat16>::value)
                 out[a * NB + b] = __float2bfloat16_rn(v);
               else

@@ -316,7 +316,7 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int b = s_idx[8 * (n0 + n) + 2 * t4 + e];
-            if (b >= 0) out[(int64_t)a * G.nb + b] = acc[n][m][2 * hh + e] * s;
+            if (b >= 0) out[(int64_t)a * G.nb + b] = scale_sum(acc[n][m][2 * hh + e], s);
           }
     }
 }
