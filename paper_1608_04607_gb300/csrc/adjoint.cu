@@ -25,8 +25,9 @@ namespace {
 constexpr int kCWarps = 4;      // warps per block in the contraction kernel
 constexpr int kManyRhs = 8;     // right-hand sides from which the lanes split over them
 
-// d/dx phi2 (see phi2_prime in node.cuh) in FP32: eleven terms of the series
-// below x = 1 (the first one left out is below 1e-9 of the sum)
+// d/dx phi2(x) = (2 - x - (x + 2) e^{-x}) / x^3 = sum_j (-1)^(j+1) (j+1) x^j / (j+3)!
+// in FP32: eleven terms of the series below x = 1, where the closed form cancels
+// (the first one left out is below 1e-9 of the sum)
 __device__ __forceinline__ float phi2_prime_row(float x) {
   if (x < 1.f) {
     const float c[11] = {-1.f / 6,          2.f / 24,          -3.f / 120,          4.f / 720,

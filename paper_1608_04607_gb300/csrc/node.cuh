@@ -380,25 +380,6 @@ __device__ inline void fill_patches(PatchSmem& S, float cos_max) {
   }
 }
 
-
-// d/dx phi2(x) = (2 - x - (x + 2) e^{-x}) / x^3 = sum_j (-1)^(j+1) (j+1) x^j / (j+3)!;
-// the series below x = 1 avoids the cancellation of the closed form.
-template <typename T>
-__device__ __forceinline__ T phi2_prime(T x) {
-  if (x < T(1)) {
-    // coefficients (-1)^(j+1) (j+1)/(j+3)!, j = 0..14
-    const T c[15] = {T(-1.0 / 6), T(2.0 / 24), T(-3.0 / 120), T(4.0 / 720), T(-5.0 / 5040), T(6.0 / 40320),
-                     T(-7.0 / 362880), T(8.0 / 3628800), T(-9.0 / 39916800), T(10.0 / 479001600),
-                     T(-11.0 / 6227020800.0), T(12.0 / 87178291200.0), T(-13.0 / 1307674368000.0),
-                     T(14.0 / 20922789888000.0), T(-15.0 / 355687428096000.0)};
-    T s = c[14];
-#pragma unroll
-    for (int i = 13; i >= 0; --i) s = c[i] + x * s;
-    return s;
-  }
-  return (T(2) - x - (x + T(2)) * exp_t<T>(-x)) / (x * x * x);
-}
-
 // k-th derivative of phi2 (k <= 3): phi2^(k)(x) = (-1)^k Int_0^1 (1-u) u^k e^{-x u} du.
 // Below x = 1 the Taylor series sum_m (-1)^(m+k) (m+k)!/(m! (m+k+2)!) x^m
 // (20 terms); above, a 16-point Gauss rule on the integral (the integrand is

@@ -10,7 +10,9 @@
 //  * the assembly of B (Eq. B4DInt with the closed form of Sec. 3.3 and the
 //    patch rule of Sec. 3.4), one block per (face pair, tile of test rows):
 //    the block's threads each own an 8 x 8 register tile, and each pass
-//    stages Z(p) and w Z(p') of up to 64 quadrature nodes in shared memory;
+//    stages Z(p) and w Z(p') of up to 64 quadrature nodes in shared memory, on
+//    FP32 FMAs for N_p = 9 and the linear spatial basis, on tensor cores from
+//    N_p = 10 on (assemble_wide_mma.cuh);
 //  * the forward application y = x0 + alpha B x (FP32 blocks, FP32 or FP64
 //    vectors), one block per operator row, a warp per test index streaming
 //    the row's three block rows with coalesced loads;
