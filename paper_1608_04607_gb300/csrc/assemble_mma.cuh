@@ -4,26 +4,30 @@
 // One warp per face pair.  Lanes evaluate one quadrature node each (row by
 // row, row_node.cuh); the block is the sum over nodes of w Z(p') Z(p)^T, an
 // N_b x N_b product over some 1,400 (N_p = 4) to 2,700 (N_p = 8) nodes.  Per pass of
-// 32 nodes each staged value x is split into two FP16 parts x = hi + lo
-// (22 significant bits) and the pass's product is three mma.sync m16n8k16
-// products, lo hi + hi lo + hi hi with FP32 accumulation, started at zero and
-// added to the FP32 sums on the CUDA cores.  So no sum on the tensor cores is
-// longer than 32 nodes (their accumulation rounds towards zero), and the
-// weights of a pass are scaled by a power of two to a maximum in [1, 2), which
-// keeps both FP16 parts away from the subnormal range whatever the mesh's
-// lengths and damping; the scale is taken out by the FMA that adds the pass.
-// Measured error against the same rule in 64 bits: 1.4e-7 (2-norm), where the
-// 1,394 sequential FP32 additions per entry of the rank-1 form gave 5.7e-7.
+// 32 nodes each staged value x is split into two FP16 parts x = hi + lo and the
+// pass's product is three mma.sync m16n8k16 products, hi hi, lo (hi + lo) and hi lo,
+// started at zero and added to the FP32 sums on the CUDA cores.
 //
-// Measured (GB300): 48,000 tets at N_p = 4 in 10.3 ms against 23.8 ms for the
-// rank-1 form on CUDA cores, 24,576 tets at N_p = 8 in 36.2 against 87.0 ms.
+// The tensor cores round their sums towards zero, which would make every entry
+// too small by a common factor, and a solve at little damping magnifies such a
+// loss some hundred times.  So hi hi is made exact: hi is a multiple of 2^-9,
+// |Z(p)| <= 1, and the weights of a pass are scaled by a power of two to a maximum
+// in [1, 2), so |w Z(p')| < 2.  All products are then multiples of 2^-18, and 32 of
+// them add up to at most 2^6 = 2^24 such units, which FP32 holds without
+// rounding.  The other two products have sums of their own, 2^-9 of it, and so has
+// their loss.  lo is rounded to nearest at 2^-22 at most, so a staged value is
+// exact to 2^-22 of its pass's largest (not of itself).  The scale is taken out by
+// the FMA that adds the pass.
+// Measured (GB300): 48,000 tets at N_p = 4 in 10.1 ms against 23.8 ms for the
+// rank-1 form on CUDA cores, 24,576 tets at N_p = 8 in 36.7 against 87.0 ms; error
+// against 64 bits (2-norm, 1,296 and 384 tets) 2.5e-7 against 5.7e-7 at N_p = 4,
+// 4.4e-7 against 8.3e-7 at N_p = 8.  (Parts split relative to each value, hi hi not
+// exact: 10.2 and 35.7 ms, every entry 7e-8 too small.)
 // What bounds it: issue and the FP32, ALU and shared-memory pipes together at
-// N_p = 4 (315 instructions per pass, 67% issue active, no pipe above 60%); at
-// N_p = 8 the latency of the MMA chains (108 MMAs of 8 cycles in a pass of
-// 1,750 cycles), with 255 registers and 8 warps per SM slightly ahead of 168
-// registers and 12 (36.2 against 36.9 ms; the other way round at N_p = 7, 11.2
-// against 10.5 ms at 10,368 tets).  More warps at N_p <= 4 gain nothing (24 per
-// SM: 10.5 ms).
+// N_p = 4; at N_p = 8 the latency of the MMA chains (108 MMAs of 8 cycles in a pass
+// of some 1,800), with 255 registers and 8 warps per SM.  N_p = 7 likewise: 11.8
+// ms at 10,368 tets, 12.4 ms with 168 registers and 12 warps.  More warps at
+// N_p <= 4 gain nothing (24 per SM: 10.5 ms).
 #pragma once
 
 #include <algorithm>
@@ -61,12 +65,16 @@ struct MmaWarp {
   alignas(16) __half pl[32 * MmaTile<NP>::LD];
 };
 
+// x + kSplitStep - kSplitStep is x rounded to a multiple of 2^-9 (|x| <= 2): FP32
+// has units of 2^-9 between 2^14 and 2^15, of which this is the middle
+constexpr float kSplitStep = 24576.f;
+
 // hi and lo FP16 parts of the values v[0..NB) of a node (x: Z(p), y: w Z(p');
 // zero up to a multiple of 8) into its four staged rows.  What the last m-tile
 // reads beyond that is left as it is: it reaches only block rows past N_b.
 template <int NB>
 __device__ __forceinline__ void stage_split(__half* ph, __half* pl, __half* qh, __half* ql, const float2* v) {
-  const float2 minus = pair(-1.f, -1.f);
+  const float2 minus = pair(-1.f, -1.f), step = pair(kSplitStep, kSplitStep), back = pair(-kSplitStep, -kSplitStep);
   auto bits = [](__half2 h) { return reinterpret_cast<const uint32_t&>(h); };
 #pragma unroll
   for (int u = 0; u < (NB + 7) / 8; ++u) {
@@ -79,11 +87,10 @@ __device__ __forceinline__ void stage_split(__half* ph, __half* pl, __half* qh, 
         continue;
       }
       const float2 s = v[b], t = b + 1 < NB ? v[b + 1 < NB ? b + 1 : b] : pair(0.f, 0.f);
-      const __half2 hp = __floats2half2_rn(s.x, t.x), hq = __floats2half2_rn(s.y, t.y);
-      const float2 fp = __half22float2(hp), fq = __half22float2(hq);
-      const float2 ds = fma2(pair(fp.x, fq.x), minus, s), dt = fma2(pair(fp.y, fq.y), minus, t);
-      h0[e] = bits(hp);
-      h1[e] = bits(hq);
+      const float2 hs = __fadd2_rn(__fadd2_rn(s, step), back), ht = __fadd2_rn(__fadd2_rn(t, step), back);
+      const float2 ds = fma2(hs, minus, s), dt = fma2(ht, minus, t);
+      h0[e] = bits(__floats2half2_rn(hs.x, ht.x));
+      h1[e] = bits(__floats2half2_rn(hs.y, ht.y));
       l0[e] = bits(__floats2half2_rn(ds.x, dt.x));
       l1[e] = bits(__floats2half2_rn(ds.y, dt.y));
     }
@@ -107,21 +114,19 @@ __device__ __forceinline__ void mma_f16(float d[4], const uint32_t a[4], uint32_
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// What the tensor cores' rounding towards zero takes off a pass's sum on average,
-// given back when the block is scaled.  hi hi runs over two MMAs, the first at
-// half the sum: 1.5 truncations of half a unit of 2^-23 / mantissa each, 1 / mantissa
-// being 0.72 on average: 6.4e-8.  Without it every entry is 7e-8 too small, and
-// solves at little damping magnify a loss common to all entries (gradients of
-// 384 tets at N_p = 6: 4.5e-6 off without it, 1.5e-6 with it, 2.8e-6 for FP32 sums in
-// sequence).  Where the three products have chains of their own, Z_0 = 1 makes hi hi
-// of column 0 exact, and nothing is given back there.
-constexpr float kTruncated = 6.4e-8f;
-__device__ __forceinline__ float scale_sum(float sum, float s) { return fmaf(sum, s, sum * s * kTruncated); }
+__device__ __forceinline__ uint32_t add_half2(uint32_t a, uint32_t b) {
+  const __half2 v = __hadd2(reinterpret_cast<const __half2&>(a), reinterpret_cast<const __half2&>(b));
+  return reinterpret_cast<const uint32_t&>(v);
+}
 
 // acc += inv * (staged Z(p'))^T (staged Z(p)) over the 32 nodes of a pass.
 // ldmatrix.trans of the node-major rows gives both operands: the A fragment
 // of (m-tile, 16 nodes) from four 8 x 8 pieces, and the B fragments of both
-// 16-node halves of an n-tile from one instruction.
+// 16-node halves of an n-tile from one instruction.  With hi + lo of Z(p) in FP16
+// as the other factor of the first of the two mixed products, lo lo is in it too.
+// An m-tile's two sums side by side, or with three m-tiles one after the other
+// over all of them, keep the fewest registers: 6.3 against 6.5 ms (10,368
+// tets, N_p = 6) and 36.7 against 38.8 ms (24,576 tets, N_p = 8) the other way round.
 template <int NP>
 __device__ __forceinline__ void pass_product(const MmaWarp<NP>& S, int lane, float inv,
                                              float (&acc)[MmaTile<NP>::NT][MmaTile<NP>::MT][4]) {
@@ -140,38 +145,53 @@ __device__ __forceinline__ void pass_product(const MmaWarp<NP>& S, int lane, flo
     }
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
-    uint32_t bh[4], bl[4];  // (nodes 0-7, 8-15, 16-23, 24-31) x 8 columns
+    uint32_t bh[4], bl[4], bs[4];  // (nodes 0-7, 8-15, 16-23, 24-31) x 8 columns
     ldsm4_trans(bh, S.ph + lane * LD + 8 * nt);
     ldsm4_trans(bl, S.pl + lane * LD + 8 * nt);
-    // independent chains: the m-tiles, or with one m-tile the three products
-    constexpr int CH = MT == 1 ? 3 : 1;
-    float t[CH][MT][4];
 #pragma unroll
-    for (int h = 0; h < CH; ++h)
+    for (int i = 0; i < 4; ++i) bs[i] = add_half2(bh[i], bl[i]);
+    auto add = [&](int mt, float2 u0, float2 u1) {
+      float* a = acc[nt][mt];
+      u0 = fma2(u0, pair(inv, inv), pair(a[0], a[1]));
+      u1 = fma2(u1, pair(inv, inv), pair(a[2], a[3]));
+      a[0] = u0.x, a[1] = u0.y, a[2] = u1.x, a[3] = u1.y;
+    };
+    if constexpr (MT <= 2) {
 #pragma unroll
-      for (int mt = 0; mt < MT; ++mt) t[h][mt][0] = t[h][mt][1] = t[h][mt][2] = t[h][mt][3] = 0.f;
+      for (int mt = 0; mt < MT; ++mt) {
+        float t[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt) mma_f16(t[0][mt], al[mt][ks], bh[2 * ks], bh[2 * ks + 1]);
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt) mma_f16(t[CH > 1 ? 1 : 0][mt], ah[mt][ks], bl[2 * ks], bl[2 * ks + 1]);
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-      for (int mt = 0; mt < MT; ++mt) mma_f16(t[CH - 1][mt], ah[mt][ks], bh[2 * ks], bh[2 * ks + 1]);
-#pragma unroll
-    for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-      for (int e = 0; e < 4; e += 2) {
-        float2 u = pair(t[0][mt][e], t[0][mt][e + 1]);
-        if constexpr (CH == 3) u = __fadd2_rn(__fadd2_rn(u, pair(t[1][mt][e], t[1][mt][e + 1])), pair(t[2][mt][e], t[2][mt][e + 1]));
-        const float2 s = fma2(u, pair(inv, inv), pair(acc[nt][mt][e], acc[nt][mt][e + 1]));
-        acc[nt][mt][e] = s.x;
-        acc[nt][mt][e + 1] = s.y;
+        for (int ks = 0; ks < 2; ++ks) {
+          mma_f16(t, ah[mt][ks], bh[2 * ks], bh[2 * ks + 1]);
+          mma_f16(u, al[mt][ks], bs[2 * ks], bs[2 * ks + 1]);
+          mma_f16(u, ah[mt][ks], bl[2 * ks], bl[2 * ks + 1]);
+        }
+        add(mt, __fadd2_rn(pair(u[0], u[1]), pair(t[0], t[1])), __fadd2_rn(pair(u[2], u[3]), pair(t[2], t[3])));
       }
+    } else {
+      float t[MT][4];
+      auto start = [&]() {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) t[mt][0] = t[mt][1] = t[mt][2] = t[mt][3] = 0.f;
+      };
+      auto product = [&](const uint32_t (&a)[MT][2][4], const uint32_t (&b)[4]) {
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+          for (int mt = 0; mt < MT; ++mt) mma_f16(t[mt], a[mt][ks], b[2 * ks], b[2 * ks + 1]);
+      };
+      auto finish = [&]() {
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) add(mt, pair(t[mt][0], t[mt][1]), pair(t[mt][2], t[mt][3]));
+      };
+      start();
+      product(ah, bh);
+      finish();
+      start();
+      product(al, bs);
+      product(ah, bl);
+      finish();
+    }
   }
 }
 
@@ -184,7 +204,7 @@ __device__ __noinline__ float moment_factor(int moment, float mu, float LO) {
 }
 
 template <int NP, typename TO>
-__global__ void __launch_bounds__(kWarps * 32, NP == 8 ? 2 : (NP == 7 ? 3 : (NP >= 5 ? 4 : 5)))
+__global__ void __launch_bounds__(kWarps * 32, NP >= 7 ? 2 : (NP >= 5 ? 4 : 5))
 assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const double* __restrict__ gl_x,
                     const double* __restrict__ gl_w, int q, float cos_max, TO* __restrict__ vals, int64_t row_stride,
                     unsigned long long* __restrict__ node_count, unsigned long long* __restrict__ counter, int moment) {
@@ -236,7 +256,7 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
           const int rl = lane / ps.per;
           const bool live = rl < ps.rows;
           const int row = base + (live ? rl : ps.rows - 1);
-          const int pi = (int)(((float)row + 0.5f) * qinv), i = row - pi * q;  // exact: row < 28 x 32
+          const int pi = (int)(((float)row + 0.5f) * qinv), i = row - pi * q;  // exact: row < 20 x 32
           RowConst rc;
           row_const(S.P.patch[pi], s_x[i], S.pc, rc);
           const float wi = live ? s_w[i] * area2 : 0.f;
@@ -277,7 +297,7 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
             for (int e = 0; e < 2; ++e) {
               const int b = 8 * nt + 2 * t4 + e;
               if (b >= NB) continue;
-              const float v = MT == 1 && b == 0 ? acc[nt][mt][2 * h + e] * s : scale_sum(acc[nt][mt][2 * h + e], s);
+              const float v = acc[nt][mt][2 * h + e] * s;
               if constexpr (std::is_same<TO, __nv_bfloat16>::value)
                 out[a * NB + b] = __float2bfloat16_rn(v);
               else

@@ -5,9 +5,10 @@
 // quadrature nodes every warp first evaluates its share of the next pass's
 // vectors into the other staging buffer (Z(p) or w Z(p') of 32 nodes, the
 // functions of a quarter of the m), then forms its part of the present pass's
-// product as in assemble_mma.cuh: FP16 hi + lo parts of both factors, three
-// mma.sync m16n8k16 products per 16 nodes started at zero for every 32 nodes,
-// whose weights are scaled by a power of two, then added to FP32 sums.  A warp
+// product as in assemble_mma.cuh: FP16 hi + lo parts of both factors, hi on a grid
+// on which the tensor cores' sums are exact, three mma.sync m16n8k16 products per
+// 16 nodes started at zero for every 32 nodes, whose weights are scaled by a power
+// of two, then added to FP32 sums.  A warp
 // owns 2 x TN tiles of 16 x 8 entries.
 //
 // The Zernike functions come m-major out of the radial recurrence, cosine and
@@ -16,7 +17,7 @@
 // the basis order.  N_p = 16 takes 3 x 2 x 200 MMAs per 32 nodes, 2,400 cycles of an
 // SM of its 6,400: the rest goes to the latencies of the recurrences and of the
 // FP16 splits in front of the barrier of each pass.  N_p = 16, 768 tets: 71.3 ms
-// by assemble_wide_kernel (FP32 FMAs), 36.9 ms.  Half of the warps evaluating
+// by assemble_wide_kernel (FP32 FMAs), 38.1 ms here.  Half of the warps evaluating
 // before their products and half after: 47.2 ms, instruction fetches.
 #pragma once
 
@@ -71,8 +72,8 @@ inline WideMma wide_mma_geometry(int Np) {
 // zernike_wide.h with its coefficients from a table (Q_n = (A rho^2 + B) Q_{n-2} +
 // C Q_{n-4}, entry s_pos[m] / 2 + (n - m) / 2, m = 0 from kRadial0 on) in a loop,
 // four steps unrolled so that conversions of several functions are in flight:
-// 36.9 ms at N_p = 16, 768 tets; 43.5 ms not unrolled, 38.5 ms unrolled over m and
-// n for each m mod 4, code that outgrows the instruction caches.
+// 36.9 ms at N_p = 16, 768 tets, when this was chosen; 43.5 ms not unrolled, 38.5 ms
+// unrolled over m and n for each m mod 4, code that outgrows the instruction caches.
 constexpr int kRadial0 = 128;
 __device__ __forceinline__ void stage_zernike(int Np, float px, float py, float s, int sub, const short* s_pos,
                                               const float4* s_rad, int r0, int rows, __half* hi, __half* lo) {
@@ -98,10 +99,9 @@ __device__ __forceinline__ void stage_zernike(int Np, float px, float py, float 
       qb = qn;
       const int pos = pos0 + k;
       if ((unsigned)pos < (unsigned)rows) {
-        const float v = qn * cr;
-        const __half h = __float2half_rn(v);
-        hi[pos] = h;
-        lo[pos] = __float2half_rn(v - __half2float(h));
+        const float v = qn * cr, h = (v + kSplitStep) - kSplitStep;
+        hi[pos] = __float2half_rn(h);
+        lo[pos] = __float2half_rn(v - h);
       }
     }
     const float t = cr * fr - ci * fi;
@@ -132,10 +132,9 @@ __device__ __forceinline__ void stage_zernike(int Np, float px, float py, float 
         qa = qb;
         qb = qn;
         const float v0 = qn * cr, v1 = qn * ci;
-        const __half2 h = __floats2half2_rn(v0, v1);
-        const float2 b = __half22float2(h);
-        *reinterpret_cast<__half2*>(ph + 2 * k) = h;
-        *reinterpret_cast<__half2*>(pl + 2 * k) = __floats2half2_rn(v0 - b.x, v1 - b.y);
+        const float h0 = (v0 + kSplitStep) - kSplitStep, h1 = (v1 + kSplitStep) - kSplitStep;
+        *reinterpret_cast<__half2*>(ph + 2 * k) = __floats2half2_rn(h0, h1);
+        *reinterpret_cast<__half2*>(pl + 2 * k) = __floats2half2_rn(v0 - h0, v1 - h1);
       }
     }
     const float t = cr * fr - ci * fi;
@@ -268,29 +267,26 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
               uint32_t bh[4], bl[4];
               ldsm4_trans(bh, ph + 8 * n);
               ldsm4_trans(bl, ph + pb + 8 * n);
-              float t[2][4];
+              uint32_t bs[4];
 #pragma unroll
-              for (int m = 0; m < 2; ++m) t[m][0] = t[m][1] = t[m][2] = t[m][3] = 0.f;
+              for (int i = 0; i < 4; ++i) bs[i] = add_half2(bh[i], bl[i]);
 #pragma unroll
-              for (int ks = 0; ks < 2; ++ks)
+              for (int m = 0; m < 2; ++m) {
+                float t[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int m = 0; m < 2; ++m) mma_f16(t[m], al[m][ks], bh[2 * ks], bh[2 * ks + 1]);
-#pragma unroll
-              for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-                for (int m = 0; m < 2; ++m) mma_f16(t[m], ah[m][ks], bl[2 * ks], bl[2 * ks + 1]);
-#pragma unroll
-              for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-                for (int m = 0; m < 2; ++m) mma_f16(t[m], ah[m][ks], bh[2 * ks], bh[2 * ks + 1]);
-#pragma unroll
-              for (int m = 0; m < 2; ++m)
+                for (int ks = 0; ks < 2; ++ks) {
+                  mma_f16(t, ah[m][ks], bh[2 * ks], bh[2 * ks + 1]);
+                  mma_f16(u, al[m][ks], bs[2 * ks], bs[2 * ks + 1]);
+                  mma_f16(u, ah[m][ks], bl[2 * ks], bl[2 * ks + 1]);
+                }
 #pragma unroll
                 for (int e = 0; e < 4; e += 2) {
-                  const float2 s = fma2(pair(t[m][e], t[m][e + 1]), pair(inv, inv), pair(acc[n][m][e], acc[n][m][e + 1]));
+                  const float2 v = __fadd2_rn(pair(u[e], u[e + 1]), pair(t[e], t[e + 1]));
+                  const float2 s = fma2(v, pair(inv, inv), pair(acc[n][m][e], acc[n][m][e + 1]));
                   acc[n][m][e] = s.x;
                   acc[n][m][e + 1] = s.y;
                 }
+              }
             }
           }
         }
@@ -316,7 +312,7 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int b = s_idx[8 * (n0 + n) + 2 * t4 + e];
-            if (b >= 0) out[(int64_t)a * G.nb + b] = scale_sum(acc[n][m][2 * hh + e], s);
+            if (b >= 0) out[(int64_t)a * G.nb + b] = acc[n][m][2 * hh + e] * s;
           }
     }
 }

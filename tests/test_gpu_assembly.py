@@ -151,3 +151,19 @@ def test_block_entries_have_no_common_loss(D, Np):
     d = a[..., :n, :n].double() - b
     assert abs(float((d * b.sign()).sum() / b.abs().sum())) <= 4.3e-8
     assert abs(float(d[..., 0, 0].sum() / b[..., 0, 0].sum())) <= 4.3e-8
+
+
+@pytest.mark.parametrize("quad_order", [7, 14])
+@pytest.mark.parametrize("Np", [2, 4, 5, 6, 7, 8])
+def test_isotropic_entries_do_not_depend_on_the_order(D, Np, quad_order):
+    """The entry (0, 0) is the sum of the node weights, whatever the order: with
+    the tensor cores' sums exact, every order adds the same numbers in the same
+    sequence.  The entries' means differ by nothing, or by the mean of FP32
+    roundings (at most 1e-7 each) over the 4,608 pairs where a compiler fuses a
+    multiplication differently: 1.5e-9, times 3."""
+    m = kuhn_cube_mesh(4, jitter=0.2, seed=7)
+    mesh = D.Mesh(m.verts, m.tets, refl=1.0)
+    kw = dict(mu=0.3, quad_order=quad_order, max_patch_deg=60.0)
+    a = D.Operator(mesh, Np, **kw).blocks()[..., 0, 0].double()
+    b = D.Operator(mesh, 0, **kw).blocks()[..., 0, 0].double()
+    assert abs(float((a - b).sum() / b.sum())) <= 4.5e-9
