@@ -65,7 +65,8 @@ contract_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const doubl
   constexpr int NB = (NP + 1) * (NP + 2) / 2, NB4 = ContractWarp<NP>::NB4, LD = NB | 1;
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   ContractWarp<NP>* smem = reinterpret_cast<ContractWarp<NP>*>(dyn_smem);
-  __shared__ float s_x[kMaxQ], s_w[kMaxQ], s_ninv[64];
+  __shared__ float s_x[kMaxQ], s_w[kMaxQ];
+  __shared__ double s_ninv[64];
   const int lane = threadIdx.x & 31;
   const int wid = threadIdx.x >> 5;
   ContractWarp<NP>& S = smem[wid];
@@ -88,7 +89,7 @@ contract_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const doubl
       const int64_t t = (int64_t)(p / 12);
       const int64_t J = 4 * t + (int64_t)((p % 12) / 3);
       for (int a = lane; a < NB4; a += 32)
-        S.lam[a] = a < NB ? (float)(lam[(int64_t)S.pc.out_row * NB + a] * (double)S.pc.scale * (double)s_ninv[a]) : 0.f;
+        S.lam[a] = a < NB ? (float)(lam[(int64_t)S.pc.out_row * NB + a] * (double)S.pc.scale * s_ninv[a]) : 0.f;
       start_regions(S.P, S.pc, cos_max, lane);
       const float mu = S.pc.mu, D3 = S.pc.D[2], area2 = 2.f * S.pc.area_src;
       float u[NB];

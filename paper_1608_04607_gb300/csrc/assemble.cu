@@ -74,7 +74,7 @@ assemble64_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const dou
   WarpSmem<NP>* smem = reinterpret_cast<WarpSmem<NP>*>(dyn_smem);
   T* s_x = reinterpret_cast<T*>(smem + kWarps);
   T* s_w = s_x + kMaxQ;
-  float* s_ninv = reinterpret_cast<float*>(s_w + kMaxQ);
+  T* s_ninv = s_w + kMaxQ;
   const int lane = threadIdx.x & 31;
   const int wid = threadIdx.x >> 5;
   WarpSmem<NP>& S = smem[wid];
@@ -169,7 +169,7 @@ assemble64_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const dou
     for (int r = 0; r < TR; ++r) {
       const int a = a0 + r;
       if (a >= NB) continue;
-      const T s = (T)pc.scale * (T)s_ninv[a];
+      const T s = (T)pc.scale * s_ninv[a];
 #pragma unroll
       for (int c = 0; c < TC; ++c) {
         const int b = b0 + c;
@@ -184,7 +184,7 @@ template <int NP>
 int launch_assemble64(const PairConst* pairs, int64_t npairs, const double* glx, const double* glw, int q,
                       float cos_max, double* vals, int64_t row_stride, unsigned long long* nodes, int moment,
                       cudaStream_t st) {
-  constexpr size_t smem = sizeof(WarpSmem<NP>) * kWarps + 2 * kMaxQ * sizeof(double) + 64 * sizeof(float);
+  constexpr size_t smem = sizeof(WarpSmem<NP>) * kWarps + (2 * kMaxQ + 64) * sizeof(double);
   static_assert(smem <= 220 * 1024, "assembly shared memory");
   DFM_CUDA_CHECK(cudaFuncSetAttribute(assemble64_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int64_t blocks = (npairs + kWarps - 1) / kWarps;

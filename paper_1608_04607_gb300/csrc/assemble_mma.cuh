@@ -17,11 +17,14 @@
 // rounding.  The other two products have sums of their own, 2^-9 of it, and so has
 // their loss.  lo is rounded to nearest at 2^-22 at most, so a staged value is
 // exact to 2^-22 of its pass's largest (not of itself).  The scale is taken out by
-// the FMA that adds the pass.
-// Measured (GB300): 48,000 tets at N_p = 4 in 10.1 ms against 23.8 ms for the
+// the FMA that adds the pass.  Entry (0, 0), the one such a solve hangs on, is the
+// sum of the weights, and is added up lane by lane beside the products: 32 sums of
+// some 45 terms lose less to rounding than one.
+//
+// Measured (GB300): 48,000 tets at N_p = 4 in 10.4 ms against 23.8 ms for the
 // rank-1 form on CUDA cores, 24,576 tets at N_p = 8 in 36.7 against 87.0 ms; error
-// against 64 bits (2-norm, 1,296 and 384 tets) 2.5e-7 against 5.7e-7 at N_p = 4,
-// 4.4e-7 against 8.3e-7 at N_p = 8.  (Parts split relative to each value, hi hi not
+// against 64 bits (2-norm, 1,296 and 384 tets) 2.4e-7 against 5.7e-7 at N_p = 4,
+// 4.3e-7 against 8.3e-7 at N_p = 8.  (Parts split relative to each value, hi hi not
 // exact: 10.2 and 35.7 ms, every entry 7e-8 too small.)
 // What bounds it: issue and the FP32, ALU and shared-memory pipes together at
 // N_p = 4; at N_p = 8 the latency of the MMA chains (108 MMAs of 8 cycles in a pass
@@ -213,16 +216,16 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
   extern __shared__ __align__(16) unsigned char dyn_smem[];
   MmaWarp<NP>* smem = reinterpret_cast<MmaWarp<NP>*>(dyn_smem);
   float* s_x = reinterpret_cast<float*>(smem + kWarps);
-  float* s_w = s_x + kMaxQ;
-  float* s_ninv = s_w + kMaxQ;
+  float2* s_w = reinterpret_cast<float2*>(s_x + kMaxQ);
+  float2* s_ninv = s_w + kMaxQ;
   const int lane = threadIdx.x & 31;
   const int wid = threadIdx.x >> 5;
   MmaWarp<NP>& S = smem[wid];
   if (threadIdx.x < q) {
     s_x[threadIdx.x] = (float)gl_x[threadIdx.x];
-    s_w[threadIdx.x] = (float)gl_w[threadIdx.x];
+    s_w[threadIdx.x] = two_floats(gl_w[threadIdx.x]);
   }
-  if (threadIdx.x < NB) s_ninv[threadIdx.x] = zernike_invnorm(threadIdx.x);
+  if (threadIdx.x < NB) s_ninv[threadIdx.x] = two_floats(zernike_invnorm(threadIdx.x));
   __syncthreads();
   const int g8 = lane >> 2, t4 = lane & 3;
   const float qinv = 1.f / (float)q;
@@ -244,6 +247,7 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
       for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) acc[nt][mt][0] = acc[nt][mt][1] = acc[nt][mt][2] = acc[nt][mt][3] = 0.f;
+      float w00 = 0.f;  // this lane's part of entry (0, 0)
       start_regions(S.P, S.pc, cos_max, lane);
       const float mu = S.pc.mu, D3 = S.pc.D[2], area2 = 2.f * S.pc.area_src;
       while (true) {
@@ -259,7 +263,7 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
           const int pi = (int)(((float)row + 0.5f) * qinv), i = row - pi * q;  // exact: row < 20 x 32
           RowConst rc;
           row_const(S.P.patch[pi], s_x[i], S.pc, rc);
-          const float wi = live ? s_w[i] * area2 : 0.f;
+          const float wi = live ? times(area2, s_w[i]) : 0.f;
           base += ps.rows;
           for (int j0 = 0; j0 < q; j0 += ps.per) {
             const int j = j0 + (lane - rl * ps.per);
@@ -267,7 +271,8 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
             const int jc = on ? j : q - 1;
             const RowNode g = row_node(rc, s_x[jc], D3, kind, S.pc);
             const float sk = moment == 0 ? phi2_row(mu * g.LO) : moment_factor(moment, mu, g.LO);
-            const float w = on ? wi * s_w[jc] * g.base * sk : 0.f;
+            const float w = on ? times(wi * g.base * sk, s_w[jc]) : 0.f;
+            w00 += w;
             // power of two that brings the pass's largest |w| into [1, 2)
             const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(w)));
             const unsigned ex = min(max(top >> 23, 1u), 253u);
@@ -281,6 +286,9 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
           }
         }
       }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) w00 += __shfl_xor_sync(0xffffffffu, w00, o);
+      if (lane == 0) acc[0][0][0] = w00;
       // epilogue: scale row a by lambda N_a / sqrt(|T_l||T_l'|) and store
       TO* out = vals + (int64_t)S.pc.out_row * row_stride + (int64_t)S.pc.slot * NB * NB;
       const float sp = S.pc.scale;
@@ -290,7 +298,7 @@ assemble_mma_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const d
         for (int h = 0; h < 2; ++h) {
           const int a = 16 * mt + g8 + 8 * h;
           if (a >= NB) continue;
-          const float s = sp * s_ninv[a];
+          const float s = times(sp, s_ninv[a]);
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -315,7 +323,7 @@ template <int NP, typename TO>
 int launch_assemble_mma(const PairConst* pairs, int64_t npairs, const double* glx, const double* glw, int q,
                         float cos_max, TO* vals, int64_t row_stride, unsigned long long* nodes, int moment,
                         cudaStream_t st) {
-  constexpr size_t smem = sizeof(MmaWarp<NP>) * kWarps + (2 * kMaxQ + 64) * sizeof(float);
+  constexpr size_t smem = sizeof(MmaWarp<NP>) * kWarps + (3 * kMaxQ + 2 * 64) * sizeof(float);
   static_assert(smem <= 220 * 1024, "assembly shared memory");
   static_assert(sizeof(MmaWarp<NP>) % 16 == 0, "16-byte aligned staging rows");
   DFM_CUDA_CHECK(

@@ -17,7 +17,7 @@
 // the basis order.  N_p = 16 takes 3 x 2 x 200 MMAs per 32 nodes, 2,400 cycles of an
 // SM of its 6,400: the rest goes to the latencies of the recurrences and of the
 // FP16 splits in front of the barrier of each pass.  N_p = 16, 768 tets: 71.3 ms
-// by assemble_wide_kernel (FP32 FMAs), 38.1 ms here.  Half of the warps evaluating
+// by assemble_wide_kernel (FP32 FMAs), 38.3 ms here.  Half of the warps evaluating
 // before their products and half after: 47.2 ms, instruction fetches.
 #pragma once
 
@@ -151,7 +151,8 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
   extern __shared__ __align__(16) __half stg[];  // [2][64][ldq] hi, lo; [2][64][ldp] hi, lo
   __shared__ PatchWarp P;
   __shared__ PairConst pc;
-  __shared__ float s_x[kMaxQ], s_w[kMaxQ], s_inv[2][2];
+  __shared__ float s_x[kMaxQ], s_inv[2][2], s_w00[2];
+  __shared__ float2 s_w[kMaxQ];
   __shared__ short s_idx[256];  // basis index of a staged position, -1 for the pad
   __shared__ short s_pos[geom::kWideMaxNp + 1];  // position of the first function of m
   __shared__ float4 s_rad[kRadial0 + geom::kWideMaxNp / 2 + 1];
@@ -164,7 +165,7 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
   if (tid < (int)(sizeof(PairConst) / 4)) reinterpret_cast<int*>(&pc)[tid] = reinterpret_cast<const int*>(pairs + blockIdx.x)[tid];
   if (tid < q) {
     s_x[tid] = (float)gl_x[tid];
-    s_w[tid] = (float)gl_w[tid];
+    s_w[tid] = two_floats(gl_w[tid]);
   }
   if (tid < 256) s_idx[tid] = -1;
   __syncthreads();
@@ -205,6 +206,7 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
 #pragma unroll
     for (int m = 0; m < 2; ++m) acc[n][m][0] = acc[n][m][1] = acc[n][m][2] = acc[n][m][3] = 0.f;
   unsigned long long pair_nodes = 0;
+  float w00 = 0.f;  // this lane's part of entry (0, 0), the sum of the weights (of its half of the nodes)
   // stages pass `pass` of the chunk's nodes: warp 4 sub + part the functions of m =
   // sub mod 4, part 0 and 1 Z(p) of nodes 0..31 and 32..63, 2 and 3 w Z(p')
   auto evaluate = [&](int pass, int nodes) {
@@ -220,7 +222,8 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
       stage_zernike(G.Np, g.px.x, g.py.x, 1.f, sub, s_pos, s_rad, 0, 256, h, h + pb);
     } else {
       const float sk = moment == 0 ? phi2_row(mu * g.LO) : moment_factor(moment, mu, g.LO);
-      const float w = k < nodes ? area2 * s_w[i] * s_w[j] * g.base * sk : 0.f;
+      const float w = k < nodes ? times(times(area2 * g.base * sk, s_w[i]), s_w[j]) : 0.f;
+      w00 += w;
       // power of two that brings the 32 nodes' largest |w| into [1, 2)
       const unsigned top = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(w)));
       const unsigned ex = min(max(top >> 23, 1u), 253u);
@@ -295,6 +298,10 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
     }
   }
   if (tid == 0 && blockIdx.y == 0) atomicAdd(node_count, pair_nodes);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) w00 += __shfl_xor_sync(0xffffffffu, w00, o);
+  if (lane == 0 && (warp == 2 || warp == 3)) s_w00[warp - 2] = w00;  // parts 2 and 3, the weights of either half
+  __syncthreads();
   // epilogue: basis order, row i scaled by lambda N_i / sqrt(|T_l||T_l'|)
   float* out = vals + (int64_t)pc.out_row * row_stride + (int64_t)pc.slot * G.nb * G.nb;
   const int g8 = lane >> 2, t4 = lane & 3;
@@ -305,14 +312,14 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
       const int r = r0 + 32 * wm + 16 * m + g8 + 8 * hh;
       const int a = r < 256 ? s_idx[r] : -1;
       if (a < 0) continue;
-      const float s = pc.scale * zernike_invnorm(a);
+      const float s = (float)((double)pc.scale * zernike_invnorm(a));
 #pragma unroll
       for (int n = 0; n < TN; ++n)
         if (n < nn)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int b = s_idx[8 * (n0 + n) + 2 * t4 + e];
-            if (b >= 0) out[(int64_t)a * G.nb + b] = acc[n][m][2 * hh + e] * s;
+            if (b >= 0) out[(int64_t)a * G.nb + b] = (a + b == 0 ? s_w00[0] + s_w00[1] : acc[n][m][2 * hh + e]) * s;
           }
     }
 }

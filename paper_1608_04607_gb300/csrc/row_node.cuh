@@ -153,6 +153,18 @@ __device__ __forceinline__ int fill_patches_warp(PatchWarp& S, float cos_max, in
   return np;
 }
 
+// v as the sum of two FP32 numbers.  What all pairs share, Gauss weights and norms, is
+// kept this way: the rounding of a pair's own constants averages out over a mesh,
+// but one common to all entries is magnified by a solve at little damping (FP32
+// weights alone add up to 3.0e-8 too much at q = 9 and 10, and 3.0e-8 too little at
+// q = 8).
+__device__ __forceinline__ float2 two_floats(double v) {
+  const float hi = (float)v;
+  return make_float2(hi, (float)(v - (double)hi));
+}
+// x v, rounded once (a rounded x hi plus x lo would often round back)
+__device__ __forceinline__ float times(float x, float2 v) { return fmaf(x, v.x, x * v.y); }
+
 // 1 / x to FP32 rounding (the approximate reciprocal and one Newton step)
 __device__ __forceinline__ float recip(float x) {
   float r = __fdividef(1.f, x);
@@ -231,7 +243,10 @@ __device__ __forceinline__ RowNode row_node(const RowConst& r, float eta, float 
   const float2 bc = fma2(e2, r.bc1, r.bc0);
   const float sA = fmaf(eta, r.a1, r.a0);
   const float r2 = fmaf(fx.x, fx.x, fmaf(fy.x, fy.x, zd.x * zd.x));
-  const float ri = rsqrtf(r2);
+  // 1 / |f| to FP32 rounding: one Newton step, r2 being within [1/4, 1].  rsqrtf alone
+  // is 4.9e-9 too small on average there, and base has its fourth power
+  float ri = rsqrtf(r2);
+  ri = fmaf(0.5f * ri, fmaf(-r2 * ri, ri, 1.f), ri);
   const bool ok = sA > 1e-30f;  // den >= s_A: its reciprocal stays finite
   const float inv = ok ? recip(sA + fmaxf(bc.x, 0.f) + fmaxf(bc.y, 0.f)) : 0.f;
   const float ri2 = ri * ri;

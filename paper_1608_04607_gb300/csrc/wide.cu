@@ -125,7 +125,7 @@ assemble_wide_kernel(const PairConst* __restrict__ pairs, const int2* __restrict
     s_w[tid] = (float)gl_w[tid];
   }
   for (int a = tid; a < G.trw; a += blockDim.x)
-    s_ninv[a] = row0 + a < NR ? zernike_invnorm((row0 + a) % NB) : 0.f;
+    s_ninv[a] = row0 + a < NR ? (float)zernike_invnorm((row0 + a) % NB) : 0.f;
   __syncthreads();  // pc, s_pos
   // w Z(p') needs orders 0..q_last
   const int q_last = NS == 1 ? order_of(min(row0 + G.trw, NB) - 1) : Np;
