@@ -5,12 +5,17 @@
 //
 // Per operator row the product is Y (NB x R) = sum over operators and the row's
 // three blocks of B X, a dense contraction.  Every FP32 operand is split into
-// two TF32 parts (hi, lo, 11 significant bits each), and
-// three mma.sync m16n8k8 products, lo hi + hi lo + hi hi, are accumulated in
-// FP32: about 22 significant bits per product.  The tensor cores' accumulation
-// rounds towards zero, so a face's hi hi products have accumulators of their
-// own (at most 6 additions long; the others are 2^-11 of them) and the faces
-// are added on the CUDA cores.
+// two TF32 parts (hi, lo, 11 significant bits each), in three mma.sync m16n8k8
+// products, lo hi + hi lo + hi hi; lo lo, at most 2^-23 of the product, is left out.
+// A solve magnifies what all results lose in common, so nothing here is rounded one
+// way more than once: x's hi part is rounded to nearest (with both chopped, lo lo is
+// positive wherever the product is: 1.5e-7 of it lost on average), and the tensor
+// cores, which round towards zero, add up eight hi hi products from zero, the rest
+// being added on the CUDA cores (chains over a block: another 2e-7 at 45 functions).
+// One truncation is left, 4.3e-8 on average at most; results are measured 8e-9 off in
+// common, 1e-7 (3 functions) to 2.7e-7 (45) with hi chopped and block-long chains,
+// at the same times: 494 against 521 us for 16 right-hand sides (24,576 tets, 45
+// functions), 111 against 104 us for one (16,464 tets, 28 functions).
 //
 // Work is taken by source tet: the four rows that tet t sends to (recv[4t + l'],
 // one contiguous row of each operator) read the same 4 NB coefficients of every
@@ -52,13 +57,20 @@ struct Ops {
   float coef[kMaxRhs][kMaxOps];
 };
 
-// hi: the top 11 significant bits of x, lo: the rest (exact, 13 bits) plus half
-// a unit of TF32's last place, which the multiplier's own truncation to TF32
-// turns into rounding to nearest.  Three instructions (cvt.rna twice takes
-// five).  An infinite x gives NaN products.
-__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+// An operator entry: hi its top 11 significant bits, lo the rest (exact, 13 bits)
+// plus half a unit of TF32's last place, which the multiplier's own truncation to
+// TF32 turns into rounding to nearest.  Three instructions (cvt.rna twice takes
+// five).
+__device__ __forceinline__ void split_entry(float x, uint32_t& hi, uint32_t& lo) {
   hi = __float_as_uint(x) & 0xffffe000u;
   lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;
+}
+// A coefficient: hi rounded to 11 significant bits, lo the rest (exact, 12 bits and
+// its sign).  What is not finite, or rounds to infinity, gives a result that is not
+// finite.
+__device__ __forceinline__ void split_coefficient(float x, uint32_t& hi, uint32_t& lo) {
+  hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+  lo = __float_as_uint(x - __uint_as_float(hi));
 }
 
 // d += A B, or d = A B
@@ -83,6 +95,32 @@ __host__ __device__ constexpr int m_tiles(int nb) { return (nb + 15) / 16; }
 // tets consumed side by side, at most: 16, 16 and 12 consumer warps for one,
 // two and three m-tiles
 __host__ __device__ constexpr int max_groups(int nb) { return m_tiles(nb) == 1 ? 4 : (m_tiles(nb) == 2 ? 2 : 1); }
+
+// s += t, two elements per instruction
+__device__ __forceinline__ void add4(float (&s)[4], const float (&t)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; e += 2) {
+    const float2 v = __fadd2_rn(make_float2(s[e], s[e + 1]), make_float2(t[e], t[e + 1]));
+    s[e] = v.x;
+    s[e + 1] = v.y;
+  }
+}
+
+// One output in FP32 FMAs: rows `blk` (a row of the three blocks of K operators
+// `stride` apart) times the coefficients x, the exit face's left out, times the operators'
+// weights.  The split parts of an infinite coefficient cancel, so outputs that are
+// not finite are formed again as written.
+__device__ __noinline__ float plain_output(const float* blk, int64_t stride, int nb, int K, const float* x, int exit_face,
+                                           const float* weight) {
+  float s = 0.f;
+  for (int k = 0; k < K; ++k)
+    for (int f = 0; f < 3; ++f)
+      for (int b = 0; b < nb; ++b) {
+        const float v = x[(f + (f >= exit_face ? 1 : 0)) * nb + b];
+        s = fmaf(blk[k * stride + f * nb * nb + b], weight ? v * weight[k] : v, s);
+      }
+  return s;
+}
 
 template <int NB, int NT, bool COMBO>
 __global__ void __launch_bounds__(32 * (kMaxProducers + 4 * m_tiles(NB) * max_groups(NB)), 1)
@@ -215,7 +253,7 @@ spmv_multi_kernel(const __grid_constant__ Ops ops, int K, int64_t row_stride, co
       for (int f = 0; f < 3; ++f) {
         const int l = f + (f >= lp ? 1 : 0);
         const float* blk = vals + f * NB * NB;
-        float th[NT][4], tl[NT][4];
+        float tl[NT][4];
 #pragma unroll
         for (int kk = 0; kk < KK; ++kk) {
           // this lane's contraction indices 8 kk + t4 and 8 kk + t4 + 4; beyond
@@ -225,7 +263,7 @@ spmv_multi_kernel(const __grid_constant__ Ops ops, int K, int64_t row_stride, co
           const float v[4] = {in0 ? p[0] : 0.f, in0 ? p[8 * NB] : 0.f, in1 ? p[4] : 0.f, in1 ? p[8 * NB + 4] : 0.f};
           uint32_t ah[4], al[4];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) split_tf32(v[e], ah[e], al[e]);
+          for (int e = 0; e < 4; ++e) split_entry(v[e], ah[e], al[e]);
 #pragma unroll
           for (int n = 0; n < NT; ++n) {
             float u0 = in0 ? xq[n][l * NB + 8 * kk] : 0.f, u1 = in1 ? xq[n][l * NB + 8 * kk + 4] : 0.f;
@@ -234,23 +272,35 @@ spmv_multi_kernel(const __grid_constant__ Ops ops, int K, int64_t row_stride, co
               u1 *= cf[n];
             }
             uint32_t xh[2], xl[2];
-            split_tf32(u0, xh[0], xl[0]);
-            split_tf32(u1, xh[1], xl[1]);
-            if (kk == 0) {
-              mma_tf32_k8_first(tl[n], al, xh);
-              mma_tf32_k8_first(th[n], ah, xh);
-            } else {
-              mma_tf32_k8(tl[n], al, xh);
-              mma_tf32_k8(th[n], ah, xh);
-            }
+            split_coefficient(u0, xh[0], xl[0]);
+            split_coefficient(u1, xh[1], xl[1]);
+            float th[4];
+            mma_tf32_k8_first(th, ah, xh);
+            if (kk == 0) mma_tf32_k8_first(tl[n], al, xh);
+            else mma_tf32_k8(tl[n], al, xh);
             mma_tf32_k8(tl[n], ah, xl);
+            add4(acc[n], th);
           }
         }
 #pragma unroll
-        for (int n = 0; n < NT; ++n)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) acc[n][e] += th[n][e] + tl[n][e];
+        for (int n = 0; n < NT; ++n) add4(acc[n], tl[n]);
       }
+    }
+    float zero = 0.f;  // NaN if an output is not finite
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) zero = fmaf(acc[n][e], 0.f, zero);
+    if (zero != 0.f) {
+#pragma unroll
+      for (int n = 0; n < NT; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int a = a0 + (e & 2 ? 8 : 0), r = 8 * n + 2 * t4 + (e & 1);
+          if (a < NB && r < R && !(fabsf(acc[n][e]) <= 3.402823466e38f))
+            acc[n][e] = plain_output(stage0 + s * stage_f + a * NB, row_stride, NB, nops,
+                                     slot0 + xs * slot_f + r * XS, lp, COMBO ? ops.coef[r] : nullptr);
+        }
     }
     __syncwarp();  // the row's stage and the tet's slot are read
     if (lane == 0) {
