@@ -109,6 +109,70 @@ inline WideAsm wide_asm_geometry(int nb, int ns = 1) {
   return g;
 }
 
+// ---- FP32 operators times several FP32 right-hand sides (spmv_multi_kernel) ----
+constexpr int kMultiMaxOps = 4;
+constexpr int kMultiMaxRhs = 16;       // per launch
+constexpr int kMultiMaxDepth = 16;     // ring depth (tets)
+constexpr int kMultiMaxProducers = 4;
+constexpr int kMultiHead = 2048;       // barriers: (4 + 1) depth full and as many empty ones
+// stride (floats) between the right-hand sides of a slot: 4 NB, made an odd
+// multiple of 4 so that eight right-hand sides fall into distinct banks
+DFM_GEOM_HD constexpr int multi_slot_stride(int nb) { return 4 * nb + (nb % 2 ? 0 : 4); }
+DFM_GEOM_HD constexpr int multi_m_tiles(int nb) { return (nb + 15) / 16; }
+// tets consumed side by side, at most: 16, 16 and 12 consumer warps for one,
+// two and three m-tiles
+DFM_GEOM_HD constexpr int multi_max_groups(int nb) {
+  return multi_m_tiles(nb) == 1 ? 4 : (multi_m_tiles(nb) == 2 ? 2 : 1);
+}
+
+struct Multi {
+  int producers, groups;   // producer warps and tet groups, each at most the ring's depth
+  int log_depth, log_slots;  // tets whose rows, and tets whose coefficients, are in flight
+  int64_t smem;
+};
+
+// The deepest ring that fits one block per SM, with two coefficient slots at
+// least, its producers and tet groups; no producers: it does not fit.
+inline Multi multi_geometry(int nb, int K, int R) {
+  const int64_t rows = 4 * K * op_row_stride(nb) * 4, slot = (int64_t)R * multi_slot_stride(nb) * 4;
+  // the last m-tile's unused rows read up to 16 rows of a block past its end
+  const int64_t fixed = kMultiHead + 16 * nb * 4, most = 226 * 1024;
+  Multi g{};
+  for (int l = 0; (1 << l) <= kMultiMaxDepth; ++l) {
+    const int lx = l > 1 ? l : 1;
+    const int64_t need = fixed + (rows << l) + (slot << lx);
+    if (need > most) break;
+    g.log_depth = l;
+    g.log_slots = lx;
+    g.producers = 1 << l < kMultiMaxProducers ? 1 << l : kMultiMaxProducers;
+    g.groups = 1 << l < multi_max_groups(nb) ? 1 << l : multi_max_groups(nb);
+    g.smem = need;
+  }
+  return g;
+}
+
+// Whether this kernel is the faster one for K operators and R right-hand sides of a
+// launch, against the pipeline that streams tiles of consecutive rows
+// (spmv_tma_kernel): from this many right-hand sides on.  Measured at 16,464 and
+// (up to 15 functions) 48,000 tets for 1 to 6 and 8 right-hand sides: this kernel's
+// time hardly depends on them, the other's grows with each, faster the larger the
+// basis; several operators take this one longer per byte, so that a single
+// right-hand side never pays there (three operators of 15 functions, 48,000 tets:
+// 331 against 245 us for one, 337 against 402 us for three; 28 functions, one operator
+// and one right-hand side: 113 against 132 us).  On small meshes a launch's latency
+// hides the difference.
+inline bool multi_faster(int nb, int K, int R) {
+  //                                   3             6             10            15
+  constexpr int from[8][4] = {{8, 6, 6, 6}, {5, 5, 3, 3}, {4, 2, 2, 2}, {3, 2, 3, 3},
+                              //       21            28            36            45
+                              {2, 2, 3, 3}, {1, 2, 2, 2}, {1, 2, 2, 2}, {1, 2, 2, 2}};
+  constexpr int nbs[8] = {3, 6, 10, 15, 21, 28, 36, 45};
+  if (K < 1 || K > kMultiMaxOps) return false;
+  for (int i = 0; i < 8; ++i)
+    if (nbs[i] == nb) return R >= from[i][K - 1] && multi_geometry(nb, K, R).producers > 0;
+  return false;
+}
+
 // ---- preconditioner hops on the low-precision copy (hop_kernel) ----
 constexpr int kHopConsumerWarps = 8;
 constexpr int kHopPasses = 2;  // consumer passes per tile when the copy rows are small

@@ -46,10 +46,12 @@ namespace {
 
 using namespace pipe;
 
-constexpr int kMaxOps = 4;
-constexpr int kMaxRhs = 16;
-constexpr int kMaxD = 16;    // ring depth (tets)
-constexpr int kHead = 2048;  // barriers: (4 + 1) kMaxD full and as many empty ones
+// ring and warps: launch_geometry.h (shared with a host-side check)
+constexpr int kMaxOps = geom::kMultiMaxOps, kMaxRhs = geom::kMultiMaxRhs, kMaxD = geom::kMultiMaxDepth;
+constexpr int kHead = geom::kMultiHead, kMaxProducers = geom::kMultiMaxProducers;
+using geom::multi_max_groups;
+using geom::multi_m_tiles;
+using geom::multi_slot_stride;
 static_assert(10 * kMaxD * 8 <= kHead, "barriers");
 
 struct Ops {
@@ -85,17 +87,6 @@ __device__ __forceinline__ void mma_tf32_k8_first(float d[4], const uint32_t a[4
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.f));
 }
 
-// stride (floats) between the right-hand sides of a slot: 4 NB, made an odd
-// multiple of 4 so that eight right-hand sides fall into distinct banks
-__host__ __device__ constexpr int slot_stride(int nb) { return 4 * nb + (nb % 2 ? 0 : 4); }
-
-// COMBO: K operators with per-right-hand-side weights; else one, weight 1
-constexpr int kMaxProducers = 4;
-__host__ __device__ constexpr int m_tiles(int nb) { return (nb + 15) / 16; }
-// tets consumed side by side, at most: 16, 16 and 12 consumer warps for one,
-// two and three m-tiles
-__host__ __device__ constexpr int max_groups(int nb) { return m_tiles(nb) == 1 ? 4 : (m_tiles(nb) == 2 ? 2 : 1); }
-
 // s += t, two elements per instruction
 __device__ __forceinline__ void add4(float (&s)[4], const float (&t)[4]) {
 #pragma unroll
@@ -122,12 +113,13 @@ __device__ __noinline__ float plain_output(const float* blk, int64_t stride, int
   return s;
 }
 
+// COMBO: K operators with per-right-hand-side weights; else one, weight 1
 template <int NB, int NT, bool COMBO>
-__global__ void __launch_bounds__(32 * (kMaxProducers + 4 * m_tiles(NB) * max_groups(NB)), 1)
+__global__ void __launch_bounds__(32 * (kMaxProducers + 4 * multi_m_tiles(NB) * multi_max_groups(NB)), 1)
 spmv_multi_kernel(const __grid_constant__ Ops ops, int K, int64_t row_stride, const int32_t* __restrict__ recv,
                   int nt, int64_t nrows, const float* __restrict__ x, const float* x0, float* y, int R,
                   float alpha, int P, int G, int logD, int logX, int reverse, int keep_from, int* __restrict__ err) {
-  constexpr int MT = m_tiles(NB), KK = (NB + 7) / 8, XS = slot_stride(NB);
+  constexpr int MT = multi_m_tiles(NB), KK = (NB + 7) / 8, XS = multi_slot_stride(NB);
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw);
   uint64_t* empty = full + 4 * kMaxD;
@@ -317,34 +309,9 @@ spmv_multi_kernel(const __grid_constant__ Ops ops, int K, int64_t row_stride, co
   }
 }
 
-struct MultiGeo {
-  int P = 0, G = 0, logD = 0, logX = 0;
-  size_t smem = 0;
-};
-
-// The deepest ring that fits one block per SM, with two coefficient slots at
-// least, its producers and tet groups; P = 0: it does not fit.
-MultiGeo multi_geometry(int nb, int K, int R) {
-  const int64_t rows = 4 * K * geom::op_row_stride(nb) * 4, slot = (int64_t)R * slot_stride(nb) * 4;
-  // the last m-tile's unused rows read up to 16 rows of a block past its end
-  const int64_t fixed = kHead + 16 * nb * 4, most = 226 * 1024;
-  MultiGeo g;
-  for (int l = 0; (1 << l) <= kMaxD; ++l) {
-    const int lx = std::max(l, 1);
-    const int64_t need = fixed + (rows << l) + (slot << lx);
-    if (need > most) break;
-    g.logD = l;
-    g.logX = lx;
-    g.P = std::min(kMaxProducers, 1 << l);
-    g.G = std::min(max_groups(nb), 1 << l);
-    g.smem = (size_t)need;
-  }
-  return g;
-}
-
 template <int NB>
 int launch_multi(const dfm_op* op, const Ops& ops, int K, bool combo, const float* x, const float* x0, float* y,
-                 int R, float alpha, const MultiGeo& g, cudaStream_t st) {
+                 int R, float alpha, const geom::Multi& g, cudaStream_t st) {
   int dev = 0, nsm = 0;
   DFM_CUDA_CHECK(cudaGetDevice(&dev));
   DFM_CUDA_CHECK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -352,13 +319,14 @@ int launch_multi(const dfm_op* op, const Ops& ops, int K, bool combo, const floa
   const int nt = (int)(op->nrows / 4);
   auto go = [&](auto kernel) -> int {
     DFM_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
-    const int grid = std::min(nt, nsm), threads = 32 * (g.P + 4 * m_tiles(NB) * g.G);
+    const int grid = std::min(nt, nsm), threads = 32 * (g.producers + 4 * multi_m_tiles(NB) * g.groups);
     // operator bytes kept in L2 for the next application, which sweeps the other way (as in spmv.cu)
     const int keep = (int)std::max<int64_t>(0, nt - (64ll << 20) / (4 * K * op->row_stride * 4));
     {
       ::dfm::KernelTimer timer_(DFM_KERNEL_SPMV, st);
       kernel<<<(unsigned)grid, threads, g.smem, st>>>(ops, K, op->row_stride, op->recv ? op->recv : op->mesh->recv,
-                                                       nt, op->nrows, x, x0, y, R, alpha, g.P, g.G, g.logD, g.logX,
+                                                       nt, op->nrows, x, x0, y, R, alpha, g.producers, g.groups,
+                                                       g.log_depth, g.log_slots,
                                                        next_sweep_direction(op->vals), keep, op->dev_err);
     }
     DFM_LAUNCHED();
@@ -371,19 +339,8 @@ int launch_multi(const dfm_op* op, const Ops& ops, int K, bool combo, const floa
 
 }  // namespace
 
-// Where this kernel is the faster one (measured on 384 to 48,000 tets against
-// the pipeline of spmv.cu, which streams tiles of consecutive rows): always from
-// 21 functions on (16,464 tets: 28 functions 105 against 173 us for one
-// right-hand side, 45 functions 239 against 301 us for one and 376 against
-// 2,681 us for 16); below, the more products per row the sooner (48,000 tets:
-// 15 functions 111 against 121 us for two right-hand sides, but 106 against 98
-// for one; 10 functions 110 against 144 us for four, 105 against 101 for two; 6
-// functions 108 against 188 us for eight, 99 against 85 for four).
 bool apply_multi_supported(const dfm_op* op, int K, int R) {
-  if (op->precision != DFM_F32 || !narrow_nb(op->nb) || op->nb < 3 || K > kMaxOps) return false;
-  const int products = K * std::min(R, kMaxRhs);
-  if (products < (op->nb >= 21 ? 1 : (op->nb == 15 ? 2 : (op->nb == 10 ? 3 : 6)))) return false;
-  return multi_geometry(op->nb, K, std::min(R, kMaxRhs)).P > 0;
+  return op->precision == DFM_F32 && geom::multi_faster(op->nb, K, std::min(R, kMaxRhs));
 }
 
 int apply_multi(const dfm_op* op, const dfm_op* const* combo_ops, int K, const double* coef, const float* x,
@@ -391,7 +348,7 @@ int apply_multi(const dfm_op* op, const dfm_op* const* combo_ops, int K, const d
   const int64_t stride = op->nrows * (int64_t)op->nb;
   for (int r0 = 0; r0 < R; r0 += kMaxRhs) {
     const int Rl = std::min(kMaxRhs, R - r0);
-    const MultiGeo g = multi_geometry(op->nb, K, Rl);
+    const geom::Multi g = geom::multi_geometry(op->nb, K, Rl);
     Ops ops{};
     for (int k = 0; k < K; ++k)
       ops.vals[k] = reinterpret_cast<const float*>(combo_ops ? combo_ops[k]->vals : op->vals);
