@@ -553,7 +553,8 @@ struct NeumannGeo {
 
 // Blocks and rows per block, or grid = 0 where the operator does not fit the
 // shared memory of one block per SM (30 MB in all), or has no FP64 blocks of
-// the narrow bases, or reflected parts.  A block takes at least 4,000 FP64
+// the narrow bases, or reflected parts, or where the device does not take that many
+// blocks at once (a context limited to some of the SMs).  A block takes at least 4,000 FP64
 // multiply-adds per term (about 1 us on its SM's two lanes, what a barrier
 // costs) before the rows are spread over more of them.
 inline NeumannGeo neumann_geometry(const Ctx& c) {
@@ -575,26 +576,45 @@ inline NeumannGeo neumann_geometry(const Ctx& c) {
   if (g.smem > 226 * 1024) g.grid = 0;
   // no more warps than elements: an idle warp's share of the sums costs FP64 issue too
   g.threads = std::min(kNeumannThreads, (g.rows_pb * op->nb + 31) / 32 * 32);
+  if (!g.grid) return g;
+  auto* kernel = g.grid == 1 ? neumann_kernel<true> : neumann_kernel<false>;
+  int dev = 0, coop = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, g.threads, g.smem) != cudaSuccess) {
+    cudaGetLastError();
+    coop = 0;
+  }
+  if (!coop || (int64_t)per_sm * c.nsm < g.grid) g.grid = 0;
   return g;
 }
 
 // x <- b + B x until |x_new - x| <= tol |x_new| (x: initial guess and result);
-// work: n doubles, partial: 4 nsm doubles and the state.  Returns DFM_OK, the
-// series' status in *status, or an error of the launch.
+// work: n doubles, partial: 4 nsm doubles and the state.  Returns DFM_OK and the
+// series' status in *status, or an error; *ran is false, and nothing has been
+// done, where the launch was refused because not all blocks fit at once.
 inline int neumann_small(const Ctx& c, const NeumannGeo& g, const double* b, double* x, double* work, double* partial,
-                         double tol, int max_iter, int* iters, int* status) {
+                         double tol, int max_iter, int* iters, int* status, bool* ran) {
   NeumannState* st = reinterpret_cast<NeumannState*>(partial + 4 * (int64_t)g.grid);
   DFM_CUDA_CHECK(cudaMemsetAsync(st, 0, sizeof(NeumannState), c.st));
   auto* kernel = g.grid == 1 ? neumann_kernel<true> : neumann_kernel<false>;
-  DFM_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
   const double* vals = reinterpret_cast<const double*>(c.op->vals);
   int64_t row_stride = c.op->row_stride;
   const int32_t* recv = c.op->recv ? c.op->recv : c.op->mesh->recv;
   int nrows = (int)c.op->nrows, nb = c.op->nb, rows_pb = g.rows_pb;
   int* err = c.op->dev_err;
   void* args[] = {&vals, &row_stride, &recv, &nrows, &nb, &rows_pb, &b, &x, &work, &tol, &max_iter, &partial, &st, &err};
-  DFM_CUDA_CHECK(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3((unsigned)g.grid),
-                                             dim3((unsigned)g.threads), args, g.smem, c.st));
+  {
+    const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3((unsigned)g.grid),
+                                                      dim3((unsigned)g.threads), args, g.smem, c.st);
+    *ran = e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported;
+    if (!*ran) {
+      cudaGetLastError();  // the refusal is dealt with
+      return DFM_OK;
+    }
+    DFM_CUDA_CHECK(e);
+  }
   DFM_LAUNCHED();
   NeumannState h;
   DFM_CUDA_CHECK(cudaMemcpyAsync(&h, st, sizeof(h), cudaMemcpyDeviceToHost, c.st));
@@ -1449,11 +1469,13 @@ int solve_impl(const dfm_op* op, const dfm_op* const* combo, int K, const double
     int rs = DFM_OK;
     if (method == DFM_SOLVE_NEUMANN) {
       // x <- rho0 + B x until |x_new - x| <= tol |x_new|
-      const NeumannGeo ng = neumann_geometry(c);
+      NeumannGeo ng = neumann_geometry(c);
       if (ng.grid) {
         int ns = DFM_OK;
-        const int r2 = neumann_small(c, ng, b, x, xold, part64, opts->tol, max_iter, &iters, &ns);
+        bool ran = false;
+        const int r2 = neumann_small(c, ng, b, x, xold, part64, opts->tol, max_iter, &iters, &ns, &ran);
         if (r2) return r2;
+        if (!ran) ng.grid = 0;  // the loop below
         if (ns == DFM_ERR_NONFINITE) rs = set_error(ns, "dfm_solve: non-finite Neumann iterate");
         if (ns == DFM_ERR_NOT_CONVERGED) rs = set_error(ns, "dfm_solve: Neumann series reached max_iter");
         // (a barrier that timed out is reported from the operator's flag below)

@@ -73,3 +73,48 @@ def test_streamed_wide_application(D, Np, R):
         y, ref = op.apply(x, **kw), op.apply(x.double(), **kw64)
         assert float((y - ref).abs().max()) <= 4e-6 * float(ref.abs().max())
     op.check_error()
+
+
+REFUSED = """
+// stands in for the CUDA runtime's call in a child process: a launch that does not fit
+extern "C" int cudaLaunchCooperativeKernel(const void*, ...) { return 720; }  // cudaErrorCooperativeLaunchTooLarge
+"""
+
+
+def test_neumann_series_where_the_launch_is_refused(D, tmp_path):
+    """A device that does not take all blocks at once (here a stand-in for the
+    runtime call that says so): the general loop solves the same system."""
+    import os
+    import shutil
+    import subprocess
+    import sys
+
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    src, lib = tmp_path / "refused.cpp", tmp_path / "librefused.so"
+    src.write_text(REFUSED)
+    subprocess.run([cxx, "-shared", "-fPIC", str(src), "-o", str(lib)], check=True)
+    prog = """
+import torch
+from paper_1608_04607_gb300 import dfm as D
+from paper_1608_04607_gb300.inputs import kuhn_cube_mesh
+out = []
+for n in (1, 3):
+    m = kuhn_cube_mesh(n, jitter=0.2 if n > 1 else 0.0, seed=8)
+    op = D.Operator(D.Mesh(m.verts, m.tets, refl=0.9), 3, mu=0.1, precision=D.F64)
+    b = D.source(op.mesh, 3, [0])
+    rho, info = op.solve(b, method=D.NEUMANN, tol=1e-10)
+    r = rho[0] - op.apply(rho[0], x0=b[0])
+    out.append((info.iters, float(r.norm() / rho.norm())))
+print(out)
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    got = []
+    for preload in ("", str(lib)):
+        env = dict(os.environ, LD_PRELOAD=preload, PYTHONPATH=root)
+        p = subprocess.run([sys.executable, "-c", prog], capture_output=True, text=True, env=env, cwd=root, timeout=300)
+        assert p.returncode == 0, p.stderr[-2000:]
+        got.append(eval(p.stdout.strip().splitlines()[-1]))
+    for (it, res), (it0, res0) in zip(*got):
+        assert it == it0 and res <= 1e-9 and res0 <= 1e-9
