@@ -508,7 +508,8 @@ int64_t dfm_autotune_report(char* buf, int64_t len);
 #define DFM_KERNEL_SPMV_T 2   /* y = x0 + alpha B^T x */
 #define DFM_KERNEL_DOT 3      /* Krylov multi-dot */
 #define DFM_KERNEL_AXPY 4     /* Krylov multi-axpy */
-#define DFM_KERNEL_SPMV64 5   /* y = x0 + alpha B x with FP64 vectors (residuals) */
+#define DFM_KERNEL_SPMV64 5   /* y = x0 + alpha B x with FP64 vectors (residuals); a whole
+                                 Neumann series where that is one launch */
 #define DFM_KERNEL_CONTRACT 6 /* fused lambda^T (dB/dmu) rho per tet */
 #define DFM_KERNEL_SPMV16 7   /* preconditioner hop on the low-precision copy */
 #define DFM_KERNEL_SPMV16_T 8 /* preconditioner hop on the transposed copy (adjoint solves) */

@@ -606,6 +606,7 @@ inline int neumann_small(const Ctx& c, const NeumannGeo& g, const double* b, dou
   int* err = c.op->dev_err;
   void* args[] = {&vals, &row_stride, &recv, &nrows, &nb, &rows_pb, &b, &x, &work, &tol, &max_iter, &partial, &st, &err};
   {
+    ::dfm::KernelTimer timer_(DFM_KERNEL_SPMV64, c.st);
     const cudaError_t e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kernel), dim3((unsigned)g.grid),
                                                       dim3((unsigned)g.threads), args, g.smem, c.st);
     *ran = e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported;

@@ -75,6 +75,23 @@ def test_streamed_wide_application(D, Np, R):
     op.check_error()
 
 
+def test_neumann_series_is_accounted_for(D):
+    """The one launch of a series is in the statistics of the applications it stands
+    for: every term takes over a microsecond, the residual after them some 6."""
+    op = operator(D, 1, 2, precision=D.F64)
+    b = D.source(op.mesh, 2, [0])
+    op.solve(b, method=D.NEUMANN, tol=1e-12)
+    D.stats_reset()
+    D.stats_enable(1)
+    try:
+        _, info = op.solve(b, method=D.NEUMANN, tol=1e-12)
+    finally:
+        D.stats_enable(0)
+    launches, ms = D.kernel_stats(5)  # DFM_KERNEL_SPMV64
+    D.stats_reset()
+    assert info.iters > 20 and launches >= 2 and ms > 1e-3 * info.iters
+
+
 REFUSED = """
 // stands in for the CUDA runtime's call in a child process: a launch that does not fit
 extern "C" int cudaLaunchCooperativeKernel(const void*, ...) { return 720; }  // cudaErrorCooperativeLaunchTooLarge
