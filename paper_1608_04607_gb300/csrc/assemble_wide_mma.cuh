@@ -26,45 +26,11 @@
 namespace dfm {
 namespace {
 
-constexpr int kWmWarps = 16;
-constexpr int kWmNodes = 64;  // nodes per pass
-// From here on this kernel assembles, below assemble_wide_kernel of wide.cu: per
-// pass the barrier and the evaluation weigh more than the products (N_p = 9 on 48
-// tets 0.85 ms there, 0.90 ms here; N_p = 10 on 162 tets 4.18 ms and 3.90 ms; N_p = 14
-// 13.1 and 9.1; N_p = 20 86 and 48).
-constexpr int kWideMmaMinNp = 10;
-
-struct WideMma {
-  int Np, nb;
-  int total;       // staged positions: the basis, m = 0 padded to an even number
-  int WM, WN, TN;  // warps over rows and columns, column tiles per warp
-  int rows;        // positions per row tile, 32 WM
-  int ntile;       // row tiles
-  int ldq, ldp;    // halves per staged node
-  int64_t smem;    // dynamic shared memory
-};
-
-// One row tile if its warps' column tiles stay within 8 (64 sums per thread),
-// else two.
-inline WideMma wide_mma_geometry(int Np) {
-  WideMma g{};
-  g.Np = Np;
-  g.nb = (Np + 1) * (Np + 2) / 2;
-  g.total = g.nb + ((Np / 2 + 1) & 1);
-  const int MT = (g.total + 15) / 16, NT = (g.total + 7) / 8;
-  for (g.ntile = 1; g.ntile <= 2; ++g.ntile) {
-    const int mt = (MT + g.ntile - 1) / g.ntile;
-    g.WM = (mt + 1) / 2;
-    g.WN = kWmWarps / g.WM;
-    g.TN = (NT + g.WN - 1) / g.WN;
-    if (g.TN <= 8) break;
-  }
-  g.rows = 32 * g.WM;
-  g.ldq = g.rows + 8;
-  g.ldp = NT % 2 ? 8 * NT : 8 * NT + 8;
-  g.smem = 2 * (int64_t)kWmNodes * (g.ldq + g.ldp) * 2 * 2;
-  return g;
-}
+// warps, nodes and tiles: launch_geometry.h (shared with a host-side check)
+constexpr int kWmWarps = geom::kWideMmaWarps;
+constexpr int kWmNodes = geom::kWideMmaNodes;  // per pass
+using geom::WideMma;
+using geom::kWideMmaMinNp;
 
 // The Zernike functions of order <= Np with |m| = sub mod 4 at (px, py), times
 // s: hi and lo FP16 parts at positions [r0, r0 + rows) of the staged order, into
@@ -327,8 +293,8 @@ assemble_wide_mma_kernel(const PairConst* __restrict__ pairs, const double* __re
 int launch_assemble_wide_mma(int Np, const PairConst* pairs, int64_t npairs, const double* glx, const double* glw,
                              int q, float cos_max, float* vals, int64_t row_stride, unsigned long long* nodes,
                              int moment, cudaStream_t st) {
-  const WideMma g = wide_mma_geometry(Np);
-  if (g.TN > 8 || g.smem > 222 * 1024)
+  const WideMma g = geom::wide_mma_geometry(Np);
+  if (g.TN < 2 || g.TN > geom::kWideMmaMaxTn || g.smem > 222 * 1024)
     return set_error(DFM_ERR_UNSUPPORTED, "dfm_assemble: wide assembly tile does not fit a block");
   auto go = [&](auto kernel) -> int {
     DFM_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
@@ -342,7 +308,6 @@ int launch_assemble_wide_mma(int Np, const PairConst* pairs, int64_t npairs, con
     return DFM_OK;
   };
   switch (g.TN) {
-    case 1: return go(assemble_wide_mma_kernel<1>);
     case 2: return go(assemble_wide_mma_kernel<2>);
     case 3: return go(assemble_wide_mma_kernel<3>);
     case 4: return go(assemble_wide_mma_kernel<4>);

@@ -109,6 +109,72 @@ inline WideAsm wide_asm_geometry(int nb, int ns = 1) {
   return g;
 }
 
+// ---- assembly of the wide bases on tensor cores (assemble_wide_mma_kernel) ----
+constexpr int kWideMmaWarps = 16;
+constexpr int kWideMmaNodes = 64;  // nodes per pass
+constexpr int kWideMmaMaxTn = 8;   // column tiles per warp: 64 sums per thread
+// From here on this kernel assembles, below assemble_wide_kernel of wide.cu: per
+// pass the barrier and the evaluation weigh more than the products (N_p = 9 on 48
+// tets 0.85 ms there, 0.90 ms here; N_p = 10 on 162 tets 4.18 ms and 3.90 ms; N_p = 14
+// 13.1 and 9.1; N_p = 20 86 and 48).
+constexpr int kWideMmaMinNp = 10;
+
+struct WideMma {
+  int Np, nb;
+  int total;       // staged positions: the basis, m = 0 padded to an even number
+  int WM, WN, TN;  // warps over rows and columns, column tiles per warp
+  int rows;        // positions per row tile, 32 WM
+  int ntile;       // row tiles
+  int ldq, ldp;    // halves per staged node
+  int64_t smem;    // dynamic shared memory
+};
+
+// One row tile if its warps' column tiles stay within kWideMmaMaxTn, else two.
+inline WideMma wide_mma_geometry(int Np) {
+  WideMma g{};
+  g.Np = Np;
+  g.nb = (Np + 1) * (Np + 2) / 2;
+  g.total = g.nb + ((Np / 2 + 1) & 1);
+  const int MT = (g.total + 15) / 16, NT = (g.total + 7) / 8;
+  for (g.ntile = 1; g.ntile <= 2; ++g.ntile) {
+    const int mt = (MT + g.ntile - 1) / g.ntile;
+    g.WM = (mt + 1) / 2;
+    g.WN = kWideMmaWarps / g.WM;
+    g.TN = (NT + g.WN - 1) / g.WN;
+    if (g.TN <= kWideMmaMaxTn) break;
+  }
+  g.rows = 32 * g.WM;
+  g.ldq = g.rows + 8;
+  g.ldp = NT % 2 ? 8 * NT : 8 * NT + 8;
+  g.smem = 2 * (int64_t)kWideMmaNodes * (g.ldq + g.ldp) * 2 * 2;
+  return g;
+}
+
+// ---- application of the wide bases' FP32 blocks (spmv_wide_tma_kernel) ----
+constexpr int kWideApplyChunk = 16;   // test indices per chunk
+constexpr int kWideApplyGroups = 2;   // groups of consumer warps, taking alternate chunks
+constexpr int kWideApplyMaxStages = 32;
+constexpr int kWideApplyMaxRhs = 8;   // right-hand sides per launch
+constexpr int kWideApplyHead = 1024;  // barriers
+
+struct WideApply {
+  int stages;        // chunks in flight, a multiple of the groups; 0: it does not fit
+  int piece;         // floats of one block's piece of a chunk, with room for the rounding to 16 bytes
+  int64_t smem;
+};
+
+inline WideApply wide_apply_geometry(int nb, int R) {
+  WideApply g{};
+  g.piece = kWideApplyChunk * nb + 4;
+  const int64_t stage = 3 * (int64_t)g.piece * 4, slots = 2 * (int64_t)R * 4 * nb * 4;
+  int64_t n = (226 * 1024 - kWideApplyHead - slots) / stage;
+  if (n > kWideApplyMaxStages) n = kWideApplyMaxStages;
+  if (nb > 16 * kWideApplyChunk || n < kWideApplyGroups) return g;  // (a lane holds one x0 per chunk half)
+  g.stages = (int)(n - n % kWideApplyGroups);
+  g.smem = kWideApplyHead + g.stages * stage + slots;
+  return g;
+}
+
 // ---- FP32 operators times several FP32 right-hand sides (spmv_multi_kernel) ----
 constexpr int kMultiMaxOps = 4;
 constexpr int kMultiMaxRhs = 16;       // per launch

@@ -355,12 +355,11 @@ spmv_wide_kernel(const float* __restrict__ vals, int64_t row_stride, const int32
 // Measured (768 tets, N_b = 153): 161 us (79% of the copy bandwidth) against 254
 // us for the kernel above, whose two block barriers per row left it at half.
 // ---------------------------------------------------------------------------
-constexpr int kWAc = 16;       // test indices per chunk (two per consumer warp)
-constexpr int kWWarps = 8;     // consumer warps of a group
-constexpr int kWGroups = 2;
-constexpr int kWMaxStages = 32;
-constexpr int kWMaxRhs = 8;    // right-hand sides per launch
-constexpr int kWHead = 1024;   // barriers
+constexpr int kWWarps = 8;  // consumer warps of a group
+// chunks, groups and stages: launch_geometry.h (shared with a host-side check)
+constexpr int kWAc = geom::kWideApplyChunk, kWGroups = geom::kWideApplyGroups;  // (two test indices per warp)
+constexpr int kWMaxStages = geom::kWideApplyMaxStages, kWMaxRhs = geom::kWideApplyMaxRhs, kWHead = geom::kWideApplyHead;
+static_assert(kWAc == 2 * kWWarps, "a warp's test indices");
 static_assert((2 * kWMaxStages + 4) * 8 <= kWHead, "barriers");
 
 __global__ void __launch_bounds__(32 * (kWGroups * kWWarps + 1), 1)
@@ -806,16 +805,15 @@ int apply_wide_tma(const dfm_op* op, const float* x, const float* x0, float* y, 
   const int64_t stride = op->nrows * (int64_t)nb;
   for (int r0 = 0; r0 < R; r0 += kWMaxRhs) {
     const int Rl = std::min(kWMaxRhs, R - r0);
-    const int64_t stage = 3 * (int64_t)(kWAc * nb + 4) * 4, slots = 2 * (int64_t)Rl * 4 * nb * 4;
-    const int stages = (int)std::min<int64_t>(kWMaxStages, (226 * 1024 - kWHead - slots) / stage) & ~1;
-    const size_t smem = kWHead + (size_t)(stages * stage + slots);
+    const geom::WideApply g = geom::wide_apply_geometry(nb, Rl);
+    if (g.stages < kWGroups) return set_error(DFM_ERR_UNSUPPORTED, "dfm_apply: wide application does not fit a block");
     const int64_t grid = std::min<int64_t>(op->nrows * cpr, device_sms());
-    DFM_CUDA_CHECK(cudaFuncSetAttribute(spmv_wide_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    DFM_CUDA_CHECK(cudaFuncSetAttribute(spmv_wide_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
     {
       ::dfm::KernelTimer timer_(DFM_KERNEL_SPMV, st);
-      spmv_wide_tma_kernel<<<(unsigned)grid, 32 * (kWGroups * kWWarps + 1), smem, st>>>(
+      spmv_wide_tma_kernel<<<(unsigned)grid, 32 * (kWGroups * kWWarps + 1), (size_t)g.smem, st>>>(
           reinterpret_cast<const float*>(op->vals), op->row_stride, recv, op->nrows, nb, x + r0 * stride,
-          x0 ? x0 + r0 * stride : nullptr, y + r0 * stride, Rl, alpha, cpr, stages, op->dev_err);
+          x0 ? x0 + r0 * stride : nullptr, y + r0 * stride, Rl, alpha, cpr, g.stages, op->dev_err);
     }
     DFM_LAUNCHED();
     DFM_CUDA_CHECK(cudaGetLastError());
