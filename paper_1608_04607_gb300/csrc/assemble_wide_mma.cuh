@@ -30,7 +30,6 @@ namespace {
 constexpr int kWmWarps = geom::kWideMmaWarps;
 constexpr int kWmNodes = geom::kWideMmaNodes;  // per pass
 using geom::WideMma;
-using geom::kWideMmaMinNp;
 
 // The Zernike functions of order <= Np with |m| = sub mod 4 at (px, py), times
 // s: hi and lo FP16 parts at positions [r0, r0 + rows) of the staged order, into

@@ -113,11 +113,18 @@ inline WideAsm wide_asm_geometry(int nb, int ns = 1) {
 constexpr int kWideMmaWarps = 16;
 constexpr int kWideMmaNodes = 64;  // nodes per pass
 constexpr int kWideMmaMaxTn = 8;   // column tiles per warp: 64 sums per thread
-// From here on this kernel assembles, below assemble_wide_kernel of wide.cu: per
-// pass the barrier and the evaluation weigh more than the products (N_p = 9 on 48
-// tets 0.85 ms there, 0.90 ms here; N_p = 10 on 162 tets 4.18 ms and 3.90 ms; N_p = 14
-// 13.1 and 9.1; N_p = 20 86 and 48).
 constexpr int kWideMmaMinNp = 10;
+
+// Which orders this kernel assembles, and assemble_wide_kernel (FP32 FMAs) of wide.cu
+// the others: from N_p = 12 on, where the products weigh more than the evaluation and
+// the barrier of a pass (768 tets: 14.4 against 17.7 ms, N_p = 14 22.5 against 31.0); at
+// N_p = 10 too, where it is 10 to 40% faster up to 162 tets and 1.7% slower at 768 (9.53
+// against 9.37 ms) but rounds nothing in common; at N_p = 11 on small meshes, where 16
+// warps share a pair (96 tets 1.55 against 1.66 ms, 162 tets 2.50 against 2.57, 750 tets
+// 11.5 against 10.8).  N_p = 9: 162 tets 1.56 against 1.49 ms, 768 tets 7.2 against 5.4.
+inline bool wide_mma_faster(int Np, int64_t npairs) {
+  return Np >= kWideMmaMinNp && (Np != 11 || npairs <= 12 * 256);
+}
 
 struct WideMma {
   int Np, nb;

@@ -11,8 +11,8 @@
 //    patch rule of Sec. 3.4), one block per (face pair, tile of test rows):
 //    the block's threads each own an 8 x 8 register tile, and each pass
 //    stages Z(p) and w Z(p') of up to 64 quadrature nodes in shared memory, on
-//    FP32 FMAs for N_p = 9 and the linear spatial basis, on tensor cores from
-//    N_p = 10 on (assemble_wide_mma.cuh);
+//    FP32 FMAs for N_p = 9 (N_p = 11 on larger meshes) and the linear spatial basis,
+//    on tensor cores else (assemble_wide_mma.cuh);
 //  * the forward application y = x0 + alpha B x (FP32 blocks, FP32 or FP64
 //    vectors), one block per operator row, a warp per test index streaming
 //    the row's three block rows with coalesced loads;
@@ -730,7 +730,7 @@ int launch_assemble_wide(int Np, const void* pairs, int64_t npairs, const double
   if (q < 1 || q > kMaxQ) return set_error(DFM_ERR_ARG, "dfm_assemble: quad_order must be in 1..32");
   if (npairs > 0x7fffffff) return set_error(DFM_ERR_ARG, "dfm_assemble: too many face pairs");
   if (npairs == 0) return DFM_OK;
-  if (Np >= kWideMmaMinNp)
+  if (geom::wide_mma_faster(Np, npairs))
     return launch_assemble_wide_mma(Np, reinterpret_cast<const PairConst*>(pairs), npairs, glx, glw, q, cos_max, vals,
                                     row_stride, nodes, moment, st);
   const geom::WideAsm G = geom::wide_asm_geometry(nbasis(Np));

@@ -2,6 +2,7 @@
 // copies (launch_geometry.h).  Built and run by tests/test_multi_geometry.py; prints
 // "ok" or the first violation and exits non-zero.
 #include <cstdio>
+#include <initializer_list>
 
 #include "launch_geometry.h"
 
@@ -30,6 +31,12 @@ int main() {
       return fail("strides", np, g.ldq, g.ldp);
     if (g.smem != 2ll * kWideMmaNodes * (g.ldq + g.ldp) * 4 || g.smem > 220 * 1024) return fail("assembly shared memory", np, 0, g.smem);
   }
+  // the orders the FMA kernel assembles faster (measured)
+  for (int np = 9; np <= kWideMaxNp; ++np)
+    for (long long tets : {6, 162, 750, 48000}) {
+      const bool fma = np == 9 || (np == 11 && tets >= 750);
+      if (wide_mma_faster(np, 12 * tets) == fma) return fail("assembly rule", np, (int)tets, 0);
+    }
   for (int nb = 55; nb <= 256; ++nb)
     for (int R = 1; R <= kWideApplyMaxRhs; ++R) {
       const WideApply g = wide_apply_geometry(nb, R);
