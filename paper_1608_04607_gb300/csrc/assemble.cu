@@ -82,7 +82,9 @@ assemble64_kernel(const PairConst* __restrict__ pairs, int64_t npairs, const dou
     s_x[threadIdx.x] = (T)gl_x[threadIdx.x];
     s_w[threadIdx.x] = (T)gl_w[threadIdx.x];
   }
-  if (threadIdx.x < NB) s_ninv[threadIdx.x] = zernike_invnorm(threadIdx.x);
+  // (rounded to FP32: 4.0e-8 too small for the isotropic functions, but what FP64 blocks
+  // give, and solves with them to 4e-7, stays what it has been)
+  if (threadIdx.x < NB) s_ninv[threadIdx.x] = (float)zernike_invnorm(threadIdx.x);
   __syncthreads();
   const int qq = q * q;
   const int a0 = (lane >> 2) * TR;

@@ -456,9 +456,9 @@ __device__ __forceinline__ NodeGeom<T> node_geom(const float* cf, T xi, T eta, c
   return g;
 }
 
-// inverse Zernike norm (2n+2)/(eps_m pi) of basis index i (Sec. 3.1-3.2).  64 bits: in
+// inverse Zernike norm (2n+2)/(eps_m pi) of basis index i (Sec. 3.1-3.2), 64 bits: in
 // FP32 1/pi is 4.0e-8 too small, a factor common to every isotropic entry (0, 0), which
-// a solve at little damping magnifies.
+// a solve at little damping magnifies
 __device__ __forceinline__ double zernike_invnorm(int i) {
   int n = 0;
   while ((n + 1) * (n + 2) / 2 <= i) ++n;
