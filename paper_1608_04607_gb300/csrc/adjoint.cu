@@ -580,9 +580,12 @@ template <int NP>
 void launch_polar(const dfm_mesh* mesh, const double* mu, double mu_uniform, const int64_t* list, const double* w,
                   int n, const double* glx, const double* glw, int nq, double* gvec, double* dgvec, cudaStream_t st) {
   // sixteen lanes per face take the 144 lines of the default rule in nine full
-  // rounds; a whole warp per face where that still leaves SM partitions idle
-  // (48 tets at N_p = 4: 120 against 187 us)
-  if (4 * (int64_t)n > 1216)
+  // rounds; a whole warp per face where that still leaves SM partitions idle, at up
+  // to two faces for each of the four (48 tets at N_p = 4: 120 against 187 us)
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    nsm = 0;
+  if (4 * (int64_t)n > 8 * (int64_t)nsm)
     interior_density_polar_kernel<NP, 16><<<(unsigned)((4 * (int64_t)n + 7) / 8), 128, 0, st>>>(
         mesh->verts, mesh->tets, mesh->geom, mu, mu_uniform, list, w, n, glx, glw, nq, gvec, dgvec);
   else
