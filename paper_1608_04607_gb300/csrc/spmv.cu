@@ -178,8 +178,14 @@ __device__ __forceinline__ void row_times_x_split_q(const TV* blk, const float2*
 // producer drains its outstanding copies (bounded) before the block exits.
 // KC = 1: a single operator (cb.K must be 1), compiled without the combination
 // loop; KC = 0: cb.K operators combined with per-right-hand-side weights.
+// Registers: 10 to 28 functions, FP32 vectors, are compiled for one block per SM
+// (left to itself the compiler may stop at 96 registers for 21 functions and load a
+// block row again for every right-hand side: 769 against 452 us for BF16 blocks and
+// 16 of them, 24,576 tets, 118 against 94 us for FP32 and one); above, more registers
+// cost a resident block (45 functions: 353 against 306 us), below they gain nothing.
 template <int NB, int KC, typename TV, typename TX, typename TA>
-__global__ void __launch_bounds__(32 * (kConsumerWarps + 1))
+__global__ void __launch_bounds__(32 * (kConsumerWarps + 1),
+                                  KC == 1 && std::is_same<TX, float>::value && NB >= 10 && NB <= 28 ? 1 : 0)
 spmv_tma_kernel(const Combo cb, int64_t row_stride, const int32_t* __restrict__ recv, int64_t nrows,
                 int rows_per_tile, int stages, const TX* __restrict__ x, const TX* x0, TX* y, int R, TA alpha,
                 int stage_x0, int reverse, int64_t keep_from, int* __restrict__ err) {
