@@ -182,6 +182,23 @@ inline WideApply wide_apply_geometry(int nb, int R) {
   return g;
 }
 
+// Where the streamed kernel is the faster one for FP32 vectors, against
+// spmv_wide_kernel (a block per operator row): from 55 functions on (below, the linear
+// spatial basis' small blocks fill neither its chunks nor its lanes) for three
+// right-hand sides or more, two from 78 functions on, one from 105 on, on meshes of
+// up to 64 tets, where a chunk is spread over more warps, always, and between with one
+// right-hand side where the measurement says so (us, streamed against row blocks: 55
+// functions, 768 tets 83 and 64 for one, 104 and 94 for two, 125 and 124 for three; 78
+// functions, 3,072 tets 340 and 308 for one, 445 and 504 for two; 91 functions 38.8 and
+// 35.7 at 162 tets, 112 and 116 at 768; 153 functions, 768 tets 175 and 266; 66
+// functions, 96 tets 27.4 and 28.4; 55 functions, 48 tets 22.3 and 25.1).
+inline bool wide_apply_faster(int nb, int R, int64_t tets) {
+  if (nb < 55 || wide_apply_geometry(nb, R < kWideApplyMaxRhs ? R : kWideApplyMaxRhs).stages == 0) return false;
+  if (R >= 3 || tets <= 64) return true;
+  if (R == 2) return nb >= 78;
+  return nb >= 105 || (nb >= 91 && tets >= 256) || (nb >= 66 && tets <= 128);
+}
+
 // ---- FP32 operators times several FP32 right-hand sides (spmv_multi_kernel) ----
 constexpr int kMultiMaxOps = 4;
 constexpr int kMultiMaxRhs = 16;       // per launch

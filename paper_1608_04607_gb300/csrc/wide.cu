@@ -822,9 +822,7 @@ int apply_wide_tma(const dfm_op* op, const float* x, const float* x0, float* y, 
 }
 
 int apply_wide(const dfm_op* op, const float* x, const float* x0, float* y, int R, double alpha, cudaStream_t st) {
-  // the streamed kernel from 55 functions on (below, the linear spatial basis'
-  // small blocks fill neither its chunks nor its lanes)
-  if (op->precision == DFM_F32 && op->nb >= 55 && op->nb <= 256)
+  if (op->precision == DFM_F32 && geom::wide_apply_faster(op->nb, R, op->nrows / 4))
     return apply_wide_tma(op, x, x0, y, R, (float)alpha, st);
   return apply_wide_t<float>(op, x, x0, y, R, alpha, st);
 }

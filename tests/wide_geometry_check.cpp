@@ -47,6 +47,18 @@ int main() {
       const long long smem = kWideApplyHead + 12ll * g.stages * g.piece + 32ll * R * nb;
       if (g.smem != smem || smem > 227 * 1024 || kWideApplyHead % 16) return fail("application shared memory", nb, R, g.smem);
     }
+  // row blocks where they are faster (measured): one right-hand side of the smaller
+  // bases, and never a basis the ring does not hold
+  for (int nb : {55, 66, 78})
+    for (long long tets : {162, 768, 3072})
+      if (wide_apply_faster(nb, 1, tets)) return fail("application rule, one", nb, (int)tets, 0);
+  for (int nb : {105, 153, 231})
+    for (long long tets : {6, 162, 768, 3072})
+      for (int R : {1, 2, 3, 8, 19})
+        if (!wide_apply_faster(nb, R, tets)) return fail("application rule", nb, (int)tets, R);
+  if (wide_apply_faster(55, 2, 768) || !wide_apply_faster(55, 3, 768) || !wide_apply_faster(55, 1, 48) ||
+      wide_apply_faster(45, 8, 768) || wide_apply_faster(257, 8, 768))
+    return fail("application rule, edges", 55, 2, 0);
   if (wide_apply_geometry(257, 1).stages || wide_apply_geometry(1 << 14, 1).stages) return fail("too large a basis", 257, 1, 0);
   std::printf("ok\n");
   return 0;
