@@ -118,12 +118,12 @@ constexpr int kWideMmaMinNp = 10;
 // Which orders this kernel assembles, and assemble_wide_kernel (FP32 FMAs) of wide.cu
 // the others: from N_p = 12 on, where the products weigh more than the evaluation and
 // the barrier of a pass (768 tets: 14.4 against 17.7 ms, N_p = 14 22.5 against 31.0); at
-// N_p = 10 too, where it is 10 to 40% faster up to 162 tets and 1.7% slower at 768 (9.53
-// against 9.37 ms) but rounds nothing in common; at N_p = 11 on small meshes, where 16
-// warps share a pair (96 tets 1.55 against 1.66 ms, 162 tets 2.50 against 2.57, 750 tets
-// 11.5 against 10.8).  N_p = 9: 162 tets 1.56 against 1.49 ms, 768 tets 7.2 against 5.4.
+// N_p = 10 and 11 on small meshes, where 16 warps share a pair (96 tets 1.27 against
+// 1.48 and 1.55 against 1.66 ms, 162 tets 2.05 against 2.29 and 2.50 against 2.57; 750
+// tets 9.36 against 9.30 and 11.5 against 10.8, 1,500 tets at N_p = 10 18.9 against
+// 18.2).  N_p = 9: 162 tets 1.56 against 1.49 ms, 768 tets 7.2 against 5.4.
 inline bool wide_mma_faster(int Np, int64_t npairs) {
-  return Np >= kWideMmaMinNp && (Np != 11 || npairs <= 12 * 256);
+  return Np >= kWideMmaMinNp && (Np >= 12 || npairs <= 12 * 256);
 }
 
 struct WideMma {

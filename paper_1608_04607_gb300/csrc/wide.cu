@@ -11,7 +11,7 @@
 //    patch rule of Sec. 3.4), one block per (face pair, tile of test rows):
 //    the block's threads each own an 8 x 8 register tile, and each pass
 //    stages Z(p) and w Z(p') of up to 64 quadrature nodes in shared memory, on
-//    FP32 FMAs for N_p = 9 (N_p = 11 on larger meshes) and the linear spatial basis,
+//    FP32 FMAs for N_p = 9 (10 and 11 on larger meshes) and the linear spatial basis,
 //    on tensor cores else (assemble_wide_mma.cuh);
 //  * the forward application y = x0 + alpha B x (FP32 blocks, FP32 or FP64
 //    vectors), one block per operator row, a warp per test index streaming

@@ -34,7 +34,7 @@ int main() {
   // the orders the FMA kernel assembles faster (measured)
   for (int np = 9; np <= kWideMaxNp; ++np)
     for (long long tets : {6, 162, 750, 48000}) {
-      const bool fma = np == 9 || (np == 11 && tets >= 750);
+      const bool fma = np == 9 || (np <= 11 && tets >= 750);
       if (wide_mma_faster(np, 12 * tets) == fma) return fail("assembly rule", np, (int)tets, 0);
     }
   for (int nb = 55; nb <= 256; ++nb)
