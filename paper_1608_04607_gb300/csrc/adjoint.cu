@@ -305,8 +305,10 @@ int launch_contract(int Np, const PairConst* pairs, int64_t npairs, const double
 //  - phi_b = Phi x_b with the Gauss nodes symmetric about Phi / 2: sine and
 //    cosine of the lower half by their series (phi <= pi / 4), of the upper half
 //    by the addition theorems.
-// Measured: 6,000 tets at N_p = 4 in 7.9 ms against 67.8 ms with every node
-// evaluated on its own.  FP64 issue bounds it.
+// Measured: 6,000 tets at N_p = 4 in 8.4 ms against 67.8 ms with every node
+// evaluated on its own.  FP64 issue bounds it: some 50 FP64 instructions per node
+// (12 for its sine and cosine, 17 for 1 / c and the exponential, 21 for the moments)
+// and 260 per line are 8.0 ms at two lanes per SM.
 // ---------------------------------------------------------------------------
 
 // coefficients of R_n^m in powers of u = 1 - 2 rho^2, after taking out one rho

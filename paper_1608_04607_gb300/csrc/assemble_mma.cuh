@@ -21,8 +21,8 @@
 // sum of the weights, and is added up lane by lane beside the products: 32 sums of
 // some 45 terms lose less to rounding than one.
 //
-// Measured (GB300): 48,000 tets at N_p = 4 in 10.4 ms against 23.8 ms for the
-// rank-1 form on CUDA cores, 24,576 tets at N_p = 8 in 36.7 against 87.0 ms; error
+// Measured (GB300): 48,000 tets at N_p = 4 in 10.5 ms against 23.8 ms for the
+// rank-1 form on CUDA cores, 24,576 tets at N_p = 8 in 37.0 against 87.0 ms; error
 // against 64 bits (2-norm, 1,296 and 384 tets) 2.4e-7 against 5.7e-7 at N_p = 4,
 // 4.3e-7 against 8.3e-7 at N_p = 8.  (Parts split relative to each value, hi hi not
 // exact: 10.2 and 35.7 ms, every entry 7e-8 too small.)

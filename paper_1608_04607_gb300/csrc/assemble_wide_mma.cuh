@@ -17,7 +17,7 @@
 // the basis order.  N_p = 16 takes 3 x 2 x 200 MMAs per 32 nodes, 2,400 cycles of an
 // SM of its 6,400: the rest goes to the latencies of the recurrences and of the
 // FP16 splits in front of the barrier of each pass.  N_p = 16, 768 tets: 71.3 ms
-// by assemble_wide_kernel (FP32 FMAs), 38.3 ms here.  Half of the warps evaluating
+// by assemble_wide_kernel (FP32 FMAs), 38.6 ms here.  Half of the warps evaluating
 // before their products and half after: 47.2 ms, instruction fetches.
 #pragma once
 
